@@ -488,9 +488,12 @@ def e2e_host(args, ix, setting, Q, steps):
 
 
 def kernel_source_sha():
-    """Hash of search.cu's code with comments and blank space removed, so that
-    counters taken on a kernel stay matched to it across comment edits."""
-    src = open(os.path.join(ROOT, "paper_1603_09320_gb300", "csrc", "search.cu")).read()
+    """Hash of the search kernel's code (search.cu and its headers) with
+    comments and blank space removed, so that counters taken on a kernel stay
+    matched to it across comment edits."""
+    files = [os.path.join(ROOT, "paper_1603_09320_gb300", "csrc", f)
+             for f in ("search.cu", "search_kernel.cuh", "search_dev.cuh")]
+    src = "\n".join(open(f).read() for f in files if os.path.exists(f))
     src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
     src = re.sub(r"//[^\n]*", " ", src)
     src = " ".join(src.split())

@@ -492,7 +492,6 @@ hnsw_status insert_layer0(hnsw_index* ix, const DevIndex& view, const std::vecto
         const uint32_t* bids = static_cast<const uint32_t*>(dbid.p) + pos;
         const uint64_t nq = uint64_t(B) * d;
         gather_rows<<<unsigned((nq + 255) / 256), 256, 0, s>>>(drows, stride, d, bids, B, static_cast<float*>(dq.p));
-        if ((e = cudaMemsetAsync(work.p, 0, 8, s)) != cudaSuccess) break;
         st = launch_search_view(ix, view, sp, static_cast<const float*>(dq.p), B, static_cast<uint32_t*>(rid.p),
                                 static_cast<float*>(rdist.p), s, static_cast<uint32_t*>(work.p));
         if (st != HNSW_OK) break;

@@ -122,8 +122,6 @@ extern "C" hnsw_status hnsw_search_noalloc(hnsw_index* ix, const float* queries,
         p += up256(ob);
     }
     if (!dd) dists = reinterpret_cast<float*>(p);
-    e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);  // the work counter starts at zero
-    if (e != cudaSuccess) return fail(HNSW_ECUDA, std::string("hnsw_search_noalloc: clear: ") + cudaGetErrorString(e));
     hnsw_search_params prm{};
     prm.k = k;
     prm.ef = ef;
