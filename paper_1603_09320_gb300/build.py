@@ -26,7 +26,8 @@ CXX_FLAGS = ["-O3", "-std=c++17", "-fPIC", "-pthread", "-I", INCLUDE, "-I", "/us
 
 SOURCES = ["search.cu", "search_f32.cu", "search_bf16.cu", "search_f16.cu", "search_fp8.cu", "search_noalloc.cu", "merge.cu", "index.cu", "stopnet.cu", "gpu_build.cu", "builder.cpp", "blob.cpp",
            "server.cpp"]
-HEADERS = ["common.hpp", "index.cuh", "stopnet.cuh", "search_dev.cuh", "search_kernel.cuh", "search_pick.cuh"]
+HEADERS = ["common.hpp", "index.cuh", "stopnet.cuh", "search_dev.cuh", "search_kernel.cuh", "search_team.cuh",
+           "search_pick.cuh"]
 
 
 def _obj(src: str) -> str:

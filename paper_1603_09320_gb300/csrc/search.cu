@@ -45,6 +45,7 @@
 #include "common.hpp"
 #include "index.cuh"
 #include "search_kernel.cuh"
+#include "search_team.cuh"
 #include "stopnet.cuh"
 
 namespace hnswgb {
@@ -259,6 +260,64 @@ void keep_pool_memory() {
 // Deferral of a launch: none, when some warp takes several queries, always.
 enum class Defer { no, automatic, always };
 
+// Warps per query of the block-per-query kernel for this search, or 0: a warp
+// per query.  The block kernel shortens a query's chain but spends more
+// instructions and registers on it, so it is taken while all queries of the
+// batch are resident at once: up to two 8-warp blocks per SM, then up to four
+// 4-warp blocks (both sides of the limits: search_team.cuh).
+int team_warps(const DevIndex& D, const hnsw_search_params& p, uint32_t n) {
+    if (p.schedule != 0 || p.check_bounds || D.N == 0 || D.N >= kTeamMaxN || std::max(p.ef, p.k) > 512) return 0;
+    const uint32_t sms = uint32_t(sm_count());
+    return n <= 2 * sms ? 8 : n <= 4 * sms ? 4 : 0;
+}
+
+// Launches the block-per-query kernel fn with nw warps per block on the
+// arguments filled in so far.
+hnsw_status launch_team(SearchArgs& a, KernelFn fn, int nw, int visited_log2, cudaStream_t s) {
+    const uint32_t slots = (std::max(a.ix.Mmax0, a.ix.Mmax) + 31u) & ~31u;
+    const size_t row32 = size_t(a.ix.row_chunks32) * 16;
+    auto layout = [&](int hl) {
+        // the visited set; after the search its bytes hold W and, for the
+        // rerank, a copy of q
+        a.hlog = hl;
+        a.off_vis = 0;
+        a.off_qs = a.efcap * 8;
+        size_t o = std::max(size_t(4) << hl, size_t(a.efcap) * 8 + (a.rerank ? row32 : 0));
+        a.off_slot = int(o);
+        o += size_t(nw) * 2 * slots * 4;
+        a.off_merge = int(o);
+        o += size_t(32 + (a.efcap <= 64 ? 64 : a.efcap <= 256 ? 256 : 512)) * 8;
+        a.off_ctl = int(o);
+        o += (sizeof(TeamCtl) + 15) & ~size_t(15);
+        return o;
+    };
+    const int sms = sm_count();
+    auto resident = [&](size_t smem) { return uint64_t(std::max(0, blocks_per_sm(fn, nw * 32, smem))) * sms; };
+    const int most = visited_log2 > 0 ? visited_log2 : std::min(14, std::max(11, ceil_log2(uint64_t(a.efp) * 32)));
+    if (layout(most) > 227 * 1024) return fail(HNSW_EINVAL, "search: ef/visited set too large for shared memory");
+    const hnsw_status st = raise_smem_limit(reinterpret_cast<const void*>(fn), layout(most), "search");
+    if (st != HNSW_OK) return st;
+    int hl = most;
+    if (visited_log2 <= 0) {
+        // the largest set that keeps as many queries resident as the smallest
+        // one does, or all of them
+        const uint64_t want = std::min<uint64_t>(a.n, resident(layout(10)));
+        while (hl > 10 && resident(layout(hl)) < want) --hl;
+    }
+    const size_t smem = layout(hl);
+    const uint64_t cap = resident(smem);
+    if (cap == 0) return fail(HNSW_ECUDA, "search: occupancy query failed");
+    const unsigned grid = unsigned(std::min<uint64_t>(a.n, cap));
+    cudaError_t e = cudaSuccess;
+    if (a.n > grid) e = cudaMemsetAsync(a.work, 0, 4, s);
+    if (e == cudaSuccess) {
+        fn<<<grid, nw * 32, smem, s>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return fail(HNSW_ECUDA, std::string("search launch: ") + cudaGetErrorString(e));
+    return HNSW_OK;
+}
+
 hnsw_status launch_search_mode(hnsw_index* ix, const hnsw_search_params& p, const float* q, uint32_t n,
                                uint32_t* ids, float* dists, hnsw_query_stats* stats, cudaStream_t s,
                                uint32_t* work, const StopModel* stop, int mode, uint64_t* ep_keys,
@@ -276,7 +335,9 @@ hnsw_status launch_search_mode(hnsw_index* ix, const hnsw_search_params& p, cons
     a.efp = p.ef > p.k ? p.ef : p.k;
     a.efcap = 1 << ceil_log2(uint64_t(a.efp < 32 ? 32 : a.efp));
     const bool stop_build = stop != nullptr && stop->period > 0;
-    const KernelFn fn = search_kernel(D, {0, stop_build, a.efcap > 64 || D.Mmax0 > 32, p.check_bounds != 0});
+    const int team = mode == 0 && !stop && defer != Defer::always ? team_warps(D, p, n) : 0;
+    const KernelFn fn = search_kernel(D, {0, stop_build, a.efcap > 64 || D.Mmax0 > 32, p.check_bounds != 0,
+                                        team ? (a.efcap <= 64 ? 2 : a.efcap <= 256 ? 8 : 16) : 0});
     if (!fn)
         return fail(HNSW_EINVAL, p.check_bounds ? "search: check_bounds is built for f32 rows of d <= 128 and bf16 of d <= 128"
                                                 : "search: unsupported row size");
@@ -303,6 +364,7 @@ hnsw_status launch_search_mode(hnsw_index* ix, const hnsw_search_params& p, cons
         a.tr_count = stop->tr_count;
         a.tr_max = stop->tr_max;
     }
+    if (team) return launch_team(a, fn, team, p.visited_log2, s);
     const size_t row32 = size_t(D.row_chunks32) * 16;
     // per-warp layout with a visited set of 2^hl slots (every piece a
     // multiple of 16 bytes); sets the offsets in t, returns the bytes

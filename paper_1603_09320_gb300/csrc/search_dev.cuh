@@ -1,5 +1,6 @@
-// search_dev.cuh -- device code of the search: launch arguments, keys, row
-// decoding and distances, the visited set, the merges into W, rerank.
+// search_dev.cuh -- device code shared by the search kernels (search.cu: one
+// warp per query; search_team.cu: a block per query): launch arguments, keys,
+// row decoding and distances, the visited set, the merges into W, rerank.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -155,6 +156,9 @@ struct SearchArgs {
     uint32_t* dfr_ctl;
     uint4* dfr_rec;  // [n]
     int dfr_hold;    // test hook: query 0's decision is never counted
+    // block-per-query kernel (search_team.cuh): byte offsets of its pieces in
+    // the block's shared memory
+    int off_vis, off_slot, off_merge, off_ctl;
     uint32_t* err;   // the index's error word (host memory mapped on the device)
 };
 
@@ -164,6 +168,7 @@ struct KernelAsk {
     bool stop;        // learned-stop checks or trace recording
     bool wide;        // W of more than 64 entries, or layer-0 lists of more than 32
     bool check;       // the bounds-checked build
+    int team_r;       // a block per query with W in 2, 8 or 16 registers per lane (0: a warp per query)
 };
 using KernelFn = void (*)(const SearchArgs);
 // the instantiation, or null when the format has none (search_f32.cu, ...)

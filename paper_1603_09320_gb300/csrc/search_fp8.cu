@@ -4,8 +4,8 @@
 namespace hnswgb {
 
 KernelFn search_kernel_fp8(const KernelAsk& k) {
-    if (k.chunks <= 8) return pick<HNSW_FP8E4M3, 8, 1, HNSW_FP8_U>(k);
-    if (k.chunks <= 32) return pick<HNSW_FP8E4M3, 32, 1, 1>(k);
+    if (k.chunks <= 8) return pick<HNSW_FP8E4M3, 8, 1, HNSW_FP8_U, 4>(k);
+    if (k.chunks <= 32) return pick<HNSW_FP8E4M3, 32, 1, 1, 4>(k);
     return nullptr;
 }
 
