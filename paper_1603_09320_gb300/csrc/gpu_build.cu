@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
@@ -49,10 +50,11 @@ using namespace hnswgb;
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxDW = 8;      // coordinates per lane: d <= 256
+constexpr int kChunk = 64;     // candidates a selection looks at together
 constexpr int kKeep = 256;     // shrink candidates examined per chunk (ascending key order)
 constexpr int kKeyBuf = 512;   // candidate keys sorted at once in a shrink
-constexpr int kMaxOld = 64;    // members of a layer-0 list (Mmax0 <= 64)
-constexpr int kWarps = 4;      // most warps per block of the selection kernels
+constexpr int kMaxOld = 64;    // members of a list (Mmax0, Mmax <= 64)
+constexpr int kWarps = 4;      // warps per block of the selection kernels
 
 __device__ __forceinline__ uint32_t f2ord(float f) {
     const uint32_t u = __float_as_uint(f);
@@ -62,151 +64,185 @@ __device__ __forceinline__ float ord2f(uint32_t o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// Per-warp shared-memory layout of the selection kernels.
-struct WarpSmem {
-    float* Rv;       // [cap][dp] vectors of the accepted elements
-    uint32_t* Rid;   // [cap]
-    float* Rd;       // [cap] their distances to the base element
-    uint32_t* Did;   // [cap] the first discarded candidates, in order (keepPrunedConnections)
-    float* Dd;       // [cap]
-    uint64_t* keys;  // [kKeyBuf] shrink candidates, (ordered distance, id)
-    uint64_t* okeys; // [kMaxOld] keys of a list's current members
-    uint32_t* cid;   // [kKeep] sorted shrink candidates
-    float* cd;       // [kKeep]
+// Shared memory of one warp's selection.
+struct SelSmem {
+    uint32_t cid[kChunk];   // the chunk's candidates
+    float cd[kChunk];
+    uint32_t live[kChunk];  // indexes of those not rejected yet, in order
+    uint32_t keep[kChunk];
+    uint32_t Rid[kMaxOld];  // accepted elements and their distances to the base
+    float Rd[kMaxOld];
+    uint32_t Did[kMaxOld];  // the first discarded candidates, in order (keepPrunedConnections)
+    float Dd[kMaxOld];
 };
 
-__host__ __device__ inline size_t warp_smem_bytes(int cap, uint32_t dp) {
-    size_t b = size_t(kKeyBuf) * 8 + size_t(kMaxOld) * 8;
-    b += size_t(cap) * dp * 4 + size_t(cap) * 16;
-    b += size_t(kKeep) * 8;
-    return (b + 15) & ~size_t(15);
-}
-
-__device__ inline WarpSmem carve(uint8_t* base, int cap, uint32_t dp) {
-    WarpSmem w;
-    uint8_t* p = base;
-    w.keys = reinterpret_cast<uint64_t*>(p);
-    p += size_t(kKeyBuf) * 8;
-    w.okeys = reinterpret_cast<uint64_t*>(p);
-    p += size_t(kMaxOld) * 8;
-    w.Rv = reinterpret_cast<float*>(p);
-    p += size_t(cap) * dp * 4;
-    w.Rid = reinterpret_cast<uint32_t*>(p);
-    p += size_t(cap) * 4;
-    w.Rd = reinterpret_cast<float*>(p);
-    p += size_t(cap) * 4;
-    w.Did = reinterpret_cast<uint32_t*>(p);
-    p += size_t(cap) * 4;
-    w.Dd = reinterpret_cast<float*>(p);
-    p += size_t(cap) * 4;
-    w.cid = reinterpret_cast<uint32_t*>(p);
-    p += size_t(kKeep) * 4;
-    w.cd = reinterpret_cast<float*>(p);
-    return w;
-}
-
-// The warp's copy of row `id`: lane l holds coordinates l, l + 32, ...
-__device__ __forceinline__ void load_vec(const float* rows, uint32_t stride, uint32_t d, uint32_t id,
-                                         float (&x)[kMaxDW], int lane) {
-    const float* r = rows + uint64_t(id) * stride;
+// A row in the registers of a team of 8 lanes: lane t holds the 16-byte chunks
+// t, t + 8, ... (coordinates 4t .. 4t+3 of every 32).
+// DW: 32-coordinate pieces per row (4: d <= 128, 8: d <= 256).
+template <int DW>
+struct TeamVec {
+    float4 v[DW];
+};
+template <int DW>
+__device__ __forceinline__ void load_team(const float* rows, uint32_t stride, uint32_t id, TeamVec<DW>& x, int lane) {
+    const float4* r = reinterpret_cast<const float4*>(rows + uint64_t(id) * stride);
 #pragma unroll
-    for (int k = 0; k < kMaxDW; ++k) {
-        const uint32_t c = uint32_t(lane + 32 * k);
-        x[k] = c < d ? __ldg(r + c) : 0.0f;
+    for (int k = 0; k < DW; ++k) {
+        const uint32_t c = uint32_t(8 * k + (lane & 7));
+        x.v[k] = 32u * k < stride && 4u * c < stride ? __ldg(r + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 }
 
-// Distance between the warp's vector x and v (shared memory, dp floats);
-// every lane returns the same value.
-__device__ __forceinline__ float dist_sm(const float (&x)[kMaxDW], const float* v, uint32_t d, int metric,
-                                         int lane) {
-    float s = 0.0f;
+// Distance between x and y, in every lane of the team.  The sum of coordinates
+// c = l (mod 32) is formed first, for every l, and these 32 sums are added as
+// a butterfly over l would (16, 8, 4, 2, 1 apart): steps 16, 8 and 4 go across
+// lanes, with half of the sums handed over at each, 2 and 1 across what the
+// lanes then hold.
+template <int DW>
+__device__ __forceinline__ float dist_team(const TeamVec<DW>& x, const TeamVec<DW>& y, int metric, int lane) {
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int k = 0; k < kMaxDW; ++k) {
-        const uint32_t c = uint32_t(lane + 32 * k);
-        if (c < d) {
+    for (int k = 0; k < DW; ++k) {  // pieces beyond the row are zero in both and add nothing
+        const float a[4] = {x.v[k].x, x.v[k].y, x.v[k].z, x.v[k].w}, b[4] = {y.v[k].x, y.v[k].y, y.v[k].z, y.v[k].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
             if (metric == HNSW_L2SQ) {
-                const float t = x[k] - v[c];
-                s = fmaf(t, t, s);
+                const float t = a[i] - b[i];
+                s[i] = fmaf(t, t, s[i]);
             } else {
-                s = fmaf(x[k], v[c], s);
+                s[i] = fmaf(a[i], b[i], s[i]);
             }
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    return metric == HNSW_L2SQ ? s : 1.0f - s;
+    const bool h4 = lane & 4, h2 = lane & 2;
+    const float u0 = (h4 ? s[2] : s[0]) + __shfl_xor_sync(kFull, h4 ? s[0] : s[2], 4);
+    const float u1 = (h4 ? s[3] : s[1]) + __shfl_xor_sync(kFull, h4 ? s[1] : s[3], 4);
+    float v = (h2 ? u1 : u0) + __shfl_xor_sync(kFull, h2 ? u0 : u1, 2);
+    v += __shfl_xor_sync(kFull, v, 1);
+    v += __shfl_xor_sync(kFull, v, 4);
+    v += __shfl_xor_sync(kFull, v, 2);
+    return metric == HNSW_L2SQ ? v : 1.0f - v;
 }
 
-// SELECT-NEIGHBORS, resumable: takes the candidates (cid[i], cd[i]), i < nc,
-// sorted by (distance to the base, id) and following every candidate of
-// earlier calls, into R (w.Rid/Rd/Rv; nr entries so far), at most cap.
+// Drops from the live candidates those that are not closer to the base than
+// to element r (strictly; Alg. 4's test); returns how many remain.
+template <int DW>
+__device__ int prune(const float* rows, uint32_t stride, int metric, uint32_t r, SelSmem& w, int na, int lane) {
+    TeamVec<DW> x;
+    load_team(rows, stride, r, x, lane);
+    const int team = lane >> 3;
+    for (int base = 0; base < na; base += 8) {  // two rows per team in flight
+        const int j0 = min(base + team, na - 1), j1 = min(base + 4 + team, na - 1);
+        const uint32_t i0 = w.live[j0], i1 = w.live[j1];
+        TeamVec<DW> y0, y1;
+        load_team(rows, stride, w.cid[i0], y0, lane);
+        load_team(rows, stride, w.cid[i1], y1, lane);
+        const float d0 = dist_team(x, y0, metric, lane), d1 = dist_team(x, y1, metric, lane);
+        if ((lane & 7) == 0) {
+            w.keep[j0] = w.cd[i0] < d0;
+            w.keep[j1] = w.cd[i1] < d1;
+        }
+    }
+    __syncwarp();
+    const bool k0 = lane < na && w.keep[lane], k1 = lane + 32 < na && w.keep[lane + 32];
+    const uint32_t v0 = k0 ? w.live[lane] : 0u, v1 = k1 ? w.live[lane + 32] : 0u;
+    const unsigned m0 = __ballot_sync(kFull, k0), m1 = __ballot_sync(kFull, k1), below = (1u << lane) - 1u;
+    if (k0) w.live[__popc(m0 & below)] = v0;
+    if (k1) w.live[__popc(m0) + __popc(m1 & below)] = v1;
+    __syncwarp();
+    return __popc(m0) + __popc(m1);
+}
+
+// SELECT-NEIGHBORS, resumable: takes the nc <= kChunk candidates in w.cid /
+// w.cd, sorted by (distance to the base, id) and following every candidate of
+// earlier calls, into R (w.Rid / Rd; nr entries so far), at most cap.
 // heuristic: Alg. 4's acceptance loop without extendCandidates (a candidate is
 // accepted when it is closer to the base than to every element accepted
 // before it, strictly); the discarded ones are recorded in order (nd so far,
-// the first cap of them: keepPrunedConnections never takes more).  Otherwise Alg. 3
-// (the cap nearest).
-__device__ void select_more(const float* rows, uint32_t stride, uint32_t d, uint32_t dp, int metric,
-                            const uint32_t* cid, const float* cd, int nc, int cap, bool heuristic,
-                            const WarpSmem& w, int& nr, int& nd, int lane) {
-    for (int i = 0; i < nc && nr < cap; ++i) {
-        const uint32_t e = cid[i];
-        const float de = cd[i];
-        bool good = true;
-        float x[kMaxDW];
-        if (heuristic) {
-            load_vec(rows, stride, d, e, x, lane);
-            for (int j = 0; j < nr; ++j)
-                if (!(de < dist_sm(x, w.Rv + size_t(j) * dp, d, metric, lane))) {
-                    good = false;
-                    break;
-                }
+// the first cap of them: keepPrunedConnections never takes more).  Otherwise
+// Alg. 3 (the cap nearest).
+// Alg. 4 asks of each candidate in turn whether an accepted element rejects
+// it; here each accepted element, in turn, rejects candidates: the next to be
+// accepted is the first one left, and the elements it is tested against are
+// those accepted before it, as in the loop.  A rejection step scores its
+// candidates 4 at a time (8 lanes each) instead of one after another, each
+// waiting for the last; a chain of at most cap steps per chunk.  Measured on
+// 1,000 elements into 20,000 (128 coordinates, efConstruction 200): a batch's
+// select_forward took 241 us and takes 97, its link_reverse 239 and 88.
+template <int DW>
+__device__ void select_more(const float* rows, uint32_t stride, int metric, int nc, int cap, bool heuristic,
+                            SelSmem& w, int& nr, int& nd, int lane) {
+    if (!heuristic) {
+        const int take = min(nc, cap - nr);
+        for (int i = lane; i < take; i += 32) {
+            w.Rid[nr + i] = w.cid[i];
+            w.Rd[nr + i] = w.cd[i];
         }
-        if (!good) {
-            if (nd < cap && lane == 0) {
-                w.Did[nd] = e;
-                w.Dd[nd] = de;
-            }
-            nd += nd < cap;
-        }
-        if (good) {
-            if (heuristic) {
-#pragma unroll
-                for (int k = 0; k < kMaxDW; ++k) {
-                    const uint32_t c = uint32_t(lane + 32 * k);
-                    if (c < dp) w.Rv[size_t(nr) * dp + c] = x[k];
-                }
-            }
-            if (lane == 0) {
-                w.Rid[nr] = e;
-                w.Rd[nr] = de;
-            }
-            ++nr;
-        }
+        nr += take;
         __syncwarp();
+        return;
     }
+    for (int i = lane; i < nc; i += 32) w.live[i] = uint32_t(i);
+    __syncwarp();
+    int na = nc;
+    for (int j = 0; j < nr && na > 0; ++j) na = prune<DW>(rows, stride, metric, w.Rid[j], w, na, lane);
+    uint64_t taken = 0;  // accepted in this chunk
+    while (na > 0 && nr < cap) {
+        const uint32_t i = w.live[0];
+        const uint32_t r = w.cid[i];
+        if (lane == 0) {
+            w.Rid[nr] = r;
+            w.Rd[nr] = w.cd[i];
+        }
+        taken |= 1ull << i;
+        ++nr;
+        __syncwarp();
+        // the rest of the list, without r itself
+        const uint32_t v0 = lane + 1 < na ? w.live[lane + 1] : 0u, v1 = lane + 33 < na ? w.live[lane + 33] : 0u;
+        __syncwarp();
+        if (lane + 1 < na) w.live[lane] = v0;
+        if (lane + 33 < na) w.live[lane + 32] = v1;
+        __syncwarp();
+        if (--na > 0 && nr < cap) na = prune<DW>(rows, stride, metric, r, w, na, lane);
+    }
+    for (int h = 0; h < nc; h += 32) {
+        const int i = h + lane;
+        const bool out = i < nc && !((taken >> i) & 1ull);
+        const unsigned m = __ballot_sync(kFull, out);
+        const int p = nd + __popc(m & ((1u << lane) - 1u));
+        if (out && p < cap) {
+            w.Did[p] = w.cid[i];
+            w.Dd[p] = w.cd[i];
+        }
+        nd = min(cap, nd + __popc(m));
+    }
+    __syncwarp();
 }
 
 // Alg. 4's last step (keepPrunedConnections): the nearest discarded
 // candidates fill R up to cap.
-__device__ void append_pruned(const WarpSmem& w, int cap, int& nr, int nd, int lane) {
-    for (int i = 0; i < nd && nr < cap; ++i) {
-        if (lane == 0) {
-            w.Rid[nr] = w.Did[i];
-            w.Rd[nr] = w.Dd[i];
-        }
-        ++nr;
+__device__ void append_pruned(SelSmem& w, int cap, int& nr, int nd, int lane) {
+    const int take = min(nd, cap - nr);
+    for (int i = lane; i < take; i += 32) {
+        w.Rid[nr + i] = w.Did[i];
+        w.Rd[nr + i] = w.Dd[i];
     }
+    nr += max(take, 0);
     __syncwarp();
 }
 
-// SELECT-NEIGHBORS over one sorted candidate list; returns |R|.
-__device__ int select_links(const float* rows, uint32_t stride, uint32_t d, uint32_t dp, int metric,
-                            const uint32_t* cid, const float* cd, int nc, int cap, bool heuristic,
-                            bool keep_pruned, const WarpSmem& w, int lane) {
+// SELECT-NEIGHBORS over a sorted candidate list (element i given by get(i, id,
+// distance)); returns |R|.
+template <int DW, class Get>
+__device__ __forceinline__ int select_links(const float* rows, uint32_t stride, int metric, Get get, int nc, int cap,
+                                            bool heuristic, bool keep_pruned, SelSmem& w, int lane) {
     int nr = 0, nd = 0;
-    select_more(rows, stride, d, dp, metric, cid, cd, nc, cap, heuristic, w, nr, nd, lane);
-    __syncwarp();
+    for (int base = 0; base < nc && nr < cap; base += kChunk) {
+        const int m = min(kChunk, nc - base);
+        for (int i = lane; i < m; i += 32) get(base + i, w.cid[i], w.cd[i]);
+        __syncwarp();
+        select_more<DW>(rows, stride, metric, m, cap, heuristic, w, nr, nd, lane);
+    }
     if (heuristic && keep_pruned) append_pruned(w, cap, nr, nd, lane);
     return nr;
 }
@@ -223,16 +259,16 @@ __global__ void gather_rows(const float* __restrict__ rows, uint32_t stride, uin
 // (dist, id), kNone-padded), written to its layer-0 row, and one reverse
 // pair per link: key = the linked element, value = the new element and their
 // distance (pairs of unused slots get key kNone).
+template <int DW>
 __global__ void __launch_bounds__(kWarps * 32) select_forward(
-    const float* __restrict__ rows, uint32_t stride, uint32_t d, uint32_t dp, int metric,
-    const uint32_t* __restrict__ bids, uint32_t B, const uint32_t* __restrict__ res_id,
+    const float* __restrict__ rows, uint32_t stride, int metric, const uint32_t* __restrict__ bids, uint32_t B, const uint32_t* __restrict__ res_id,
     const float* __restrict__ res_d, int efc, int M, int heuristic, int keep_pruned, uint32_t* __restrict__ nbr0,
     uint32_t s0, uint32_t* __restrict__ pkey, uint32_t* __restrict__ pval, float* __restrict__ pdist) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const uint32_t b = blockIdx.x * nw + wib;
+    __shared__ SelSmem sel[kWarps];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const uint32_t b = blockIdx.x * kWarps + wib;
     if (b >= B) return;
-    const WarpSmem w = carve(smem + wib * warp_smem_bytes(M, dp), M, dp);
+    SelSmem& w = sel[wib];
     const uint32_t q = bids[b];
     const uint32_t* cid = res_id + uint64_t(b) * efc;
     const float* cd = res_d + uint64_t(b) * efc;
@@ -241,8 +277,13 @@ __global__ void __launch_bounds__(kWarps * 32) select_forward(
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nc += __shfl_xor_sync(kFull, nc, o);
     // results are sorted with the kNone padding last; q itself is never reachable
-    const int nr = select_links(rows, stride, d, dp, metric, cid, cd, nc, M, heuristic != 0, keep_pruned != 0, w,
-                                lane);
+    const int nr = select_links<DW>(
+        rows, stride, metric,
+        [&](int i, uint32_t& id, float& dist) {
+            id = cid[i];
+            dist = cd[i];
+        },
+        nc, M, heuristic != 0, keep_pruned != 0, w, lane);
     for (int j = lane; j < M; j += 32) {
         const uint64_t o = uint64_t(b) * M + j;
         if (j < nr) {
@@ -294,15 +335,20 @@ __device__ __forceinline__ unsigned lanes_below(int lane) { return (1u << lane) 
 // that order is walked in chunks of kKeep: each chunk is the kKeep smallest
 // keys above the previous chunk's last one (keys are distinct: ids are),
 // found by one pass over the candidates that sorts kKeyBuf keys at a time.
+template <int DW>
 __global__ void __launch_bounds__(kWarps * 32) link_reverse(
-    const float* __restrict__ rows, uint32_t stride, uint32_t d, uint32_t dp, int metric,
-    const uint32_t* __restrict__ skey, const uint32_t* __restrict__ sidx, uint32_t npairs,
+    const float* __restrict__ rows, uint32_t stride, int metric, const uint32_t* __restrict__ skey,
+    const uint32_t* __restrict__ sidx, uint32_t npairs,
     const uint32_t* __restrict__ seg, const uint32_t* __restrict__ nseg, const uint32_t* __restrict__ pval,
     const float* __restrict__ pdist, uint32_t* __restrict__ nbr0, uint32_t s0, int Mmax0, int heuristic,
     int keep_pruned) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const WarpSmem w = carve(smem + wib * warp_smem_bytes(Mmax0, dp), Mmax0, dp);
+    __shared__ SelSmem sel[kWarps];
+    __shared__ uint64_t key_buf[kWarps][kKeyBuf];
+    __shared__ uint64_t old_keys[kWarps][kMaxOld];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = kWarps;
+    SelSmem& w = sel[wib];
+    uint64_t* keys = key_buf[wib];    // shrink candidates, (ordered distance, id)
+    uint64_t* okeys = old_keys[wib];  // keys of the list's current members
     const uint32_t nsegs = *nseg;
     for (uint32_t s = blockIdx.x * nw + wib; s < nsegs; s += gridDim.x * nw) {
         const uint32_t i0 = seg[s];
@@ -321,28 +367,17 @@ __global__ void __launch_bounds__(kWarps * 32) link_reverse(
             continue;
         }
         // keys of the current members (their distances to e recomputed)
-        float x[kMaxDW];
-        load_vec(rows, stride, d, e, x, lane);
-        for (int j = 0; j < n0; ++j) {
-            const uint32_t c = row[j];
-            float y[kMaxDW];
-            load_vec(rows, stride, d, c, y, lane);
-            float sacc = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kMaxDW; ++k) {
-                if (uint32_t(lane + 32 * k) < d) {
-                    if (metric == HNSW_L2SQ) {
-                        const float t = x[k] - y[k];
-                        sacc = fmaf(t, t, sacc);
-                    } else {
-                        sacc = fmaf(x[k], y[k], sacc);
-                    }
-                }
+        {
+            TeamVec<DW> x;
+            load_team(rows, stride, e, x, lane);
+            for (int j0 = 0; j0 < n0; j0 += 4) {
+                const int j = min(j0 + (lane >> 3), n0 - 1);
+                const uint32_t c = row[j];
+                TeamVec<DW> y;
+                load_team(rows, stride, c, y, lane);
+                const float dc = dist_team(x, y, metric, lane);
+                if ((lane & 7) == 0) okeys[j] = (uint64_t(f2ord(dc)) << 32) | c;
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(kFull, sacc, o);
-            const float dc = metric == HNSW_L2SQ ? sacc : 1.0f - sacc;
-            if (lane == 0) w.okeys[j] = (uint64_t(f2ord(dc)) << 32) | c;
         }
         __syncwarp();
         const int total = n0 + nin;
@@ -356,40 +391,42 @@ __global__ void __launch_bounds__(kWarps * 32) link_reverse(
                 const int j = b0 + lane;
                 uint64_t k = ~0ull;
                 if (j < n0) {
-                    k = w.okeys[j];
+                    k = okeys[j];
                 } else if (j < total) {
                     const uint32_t pi = sidx[i0 + uint32_t(j - n0)];
                     k = (uint64_t(f2ord(pdist[pi])) << 32) | pval[pi];
                 }
                 const bool ok = j < total && (first || k > last);
                 const unsigned m = __ballot_sync(kFull, ok);
-                if (ok) w.keys[nk + __popc(m & lanes_below(lane))] = k;
+                if (ok) keys[nk + __popc(m & lanes_below(lane))] = k;
                 nk += __popc(m);
                 if (nk > kKeyBuf - 32) {  // full: keep the kKeep smallest
-                    for (int u = nk + lane; u < kKeyBuf; u += 32) w.keys[u] = ~0ull;
+                    for (int u = nk + lane; u < kKeyBuf; u += 32) keys[u] = ~0ull;
                     __syncwarp();
-                    sort_keys(w.keys, kKeyBuf, lane);
+                    sort_keys(keys, kKeyBuf, lane);
                     nk = kKeep;
                 }
                 __syncwarp();
             }
             int n2 = 32;
             while (n2 < nk) n2 <<= 1;
-            for (int u = nk + lane; u < n2; u += 32) w.keys[u] = ~0ull;
+            for (int u = nk + lane; u < n2; u += 32) keys[u] = ~0ull;
             __syncwarp();
-            sort_keys(w.keys, n2, lane);
+            sort_keys(keys, n2, lane);
             nk = min(nk, kKeep);
             if (nk == 0) break;
-            for (int u = lane; u < nk; u += 32) {
-                w.cid[u] = uint32_t(w.keys[u] & 0xffffffffu);
-                w.cd[u] = ord2f(uint32_t(w.keys[u] >> 32));
+            for (int base = 0; base < nk && nr < Mmax0; base += kChunk) {
+                const int m = min(kChunk, nk - base);
+                for (int i = lane; i < m; i += 32) {
+                    w.cid[i] = uint32_t(keys[base + i] & 0xffffffffu);
+                    w.cd[i] = ord2f(uint32_t(keys[base + i] >> 32));
+                }
+                __syncwarp();
+                select_more<DW>(rows, stride, metric, m, Mmax0, heuristic != 0, w, nr, nd, lane);
             }
-            __syncwarp();
-            select_more(rows, stride, d, dp, metric, w.cid, w.cd, nk, Mmax0, heuristic != 0, w, nr, nd, lane);
-            __syncwarp();
             seen += nk;
             if (nr >= Mmax0 || seen >= total) break;
-            last = w.keys[nk - 1];
+            last = keys[nk - 1];
             first = false;
             __syncwarp();
         }
@@ -425,7 +462,7 @@ hnsw_status insert_layer0(hnsw_index* ix, const DevIndex& view, const std::vecto
     if (ids.empty()) return HNSW_OK;
     const DevIndex& D = view;
     const float* drows = reinterpret_cast<const float*>(D.vec);
-    const uint32_t d = D.d, stride = D.row_chunks * 4, dp = D.row_chunks * 4, s0 = D.s0;
+    const uint32_t d = D.d, stride = D.row_chunks * 4, s0 = D.s0;
     uint32_t* nbr0 = const_cast<uint32_t*>(D.nbr0);
     const uint32_t Bmax = uint32_t(std::min<uint64_t>(32768, std::max<uint64_t>(64, ids.size())));
     DevBuf dbid, dq, rid, rdist, pkey, pval, pdist, skey, sidx, idx, seg, nseg, work, tmp;
@@ -462,23 +499,7 @@ hnsw_status insert_layer0(hnsw_index* ix, const DevIndex& view, const std::vecto
     if ((e = cudaMemcpyAsync(idx.p, iota.data(), size_t(npair_max) * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(dbid.p, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return cuda_fail(e, "copy");
-    // warps per block: as many (up to kWarps) as the shared memory allows
-    auto warps_for = [](size_t per_warp) {
-        int nw = kWarps;
-        while (nw > 1 && size_t(nw) * per_warp > 227 * 1024) --nw;
-        return nw;
-    };
-    const int fw_w = warps_for(warp_smem_bytes(M, dp)), rv_w = warps_for(warp_smem_bytes(Mmax0, dp));
-    const size_t fw_smem = size_t(fw_w) * warp_smem_bytes(M, dp);
-    const size_t rv_smem = size_t(rv_w) * warp_smem_bytes(Mmax0, dp);
-    if (fw_smem > 227 * 1024 || rv_smem > 227 * 1024)
-        return fail(HNSW_EINVAL, "layer-0 insertion: dimension too large for the selection kernels");
-    {
-        hnsw_status r = raise_smem_limit(reinterpret_cast<const void*>(select_forward), fw_smem, "layer-0 insertion");
-        if (r == HNSW_OK)
-            r = raise_smem_limit(reinterpret_cast<const void*>(link_reverse), rv_smem, "layer-0 insertion");
-        if (r != HNSW_OK) return r;
-    }
+    const bool wide = stride > 128;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -495,8 +516,8 @@ hnsw_status insert_layer0(hnsw_index* ix, const DevIndex& view, const std::vecto
         st = launch_search_view(ix, view, sp, static_cast<const float*>(dq.p), B, static_cast<uint32_t*>(rid.p),
                                 static_cast<float*>(rdist.p), s, static_cast<uint32_t*>(work.p));
         if (st != HNSW_OK) break;
-        select_forward<<<(B + fw_w - 1) / fw_w, fw_w * 32, fw_smem, s>>>(
-            drows, stride, d, dp, metric, bids, B, static_cast<const uint32_t*>(rid.p),
+        (wide ? select_forward<8> : select_forward<4>)<<<(B + kWarps - 1) / kWarps, kWarps * 32, 0, s>>>(
+            drows, stride, metric, bids, B, static_cast<const uint32_t*>(rid.p),
             static_cast<const float*>(rdist.p), efc, M, heuristic, keep_pruned, nbr0, s0,
             static_cast<uint32_t*>(pkey.p), static_cast<uint32_t*>(pval.p), static_cast<float*>(pdist.p));
         const uint32_t np = B * uint32_t(M);
@@ -508,8 +529,8 @@ hnsw_status insert_layer0(hnsw_index* ix, const DevIndex& view, const std::vecto
         if ((e = cudaMemsetAsync(nseg.p, 0, 4, s)) != cudaSuccess) break;
         mark_segments<<<(np + 255) / 256, 256, 0, s>>>(static_cast<const uint32_t*>(skey.p), np,
                                                       static_cast<uint32_t*>(seg.p), static_cast<uint32_t*>(nseg.p));
-        link_reverse<<<unsigned(sms) * 4, rv_w * 32, rv_smem, s>>>(
-            drows, stride, d, dp, metric, static_cast<const uint32_t*>(skey.p), static_cast<const uint32_t*>(sidx.p),
+        (wide ? link_reverse<8> : link_reverse<4>)<<<unsigned(sms) * 4, kWarps * 32, 0, s>>>(
+            drows, stride, metric, static_cast<const uint32_t*>(skey.p), static_cast<const uint32_t*>(sidx.p),
             np, static_cast<const uint32_t*>(seg.p), static_cast<const uint32_t*>(nseg.p),
             static_cast<const uint32_t*>(pval.p), static_cast<const float*>(pdist.p), nbr0, s0, Mmax0, heuristic,
             keep_pruned);
@@ -642,79 +663,8 @@ __device__ __forceinline__ uint64_t mkkey(float d, uint32_t id) { return (uint64
 __device__ __forceinline__ uint32_t kid(uint64_t k) { return uint32_t(k & 0xffffffffu); }
 __device__ __forceinline__ float kdist(uint64_t k) { return ord2f(uint32_t(k >> 32)); }
 
-// distance from the warp's vector x to row `id` (every lane returns it)
-__device__ __forceinline__ float dist_id(const float (&x)[kMaxDW], const float* rows, uint32_t stride, uint32_t d,
-                                         uint32_t id, int metric, int lane) {
-    float y[kMaxDW];
-    load_vec(rows, stride, d, id, y, lane);
-    float s = 0.0f;
-#pragma unroll
-    for (int k = 0; k < kMaxDW; ++k) {
-        if (uint32_t(lane + 32 * k) < d) {
-            if (metric == HNSW_L2SQ) {
-                const float t = x[k] - y[k];
-                s = fmaf(t, t, s);
-            } else {
-                s = fmaf(x[k], y[k], s);
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    return metric == HNSW_L2SQ ? s : 1.0f - s;
-}
-
-// distance from the vector a (shared memory, 16-byte aligned, d floats) to
-// row `id`, computed by one lane
-__device__ __forceinline__ float dist_lane(const float* a, const float* rows, uint32_t stride, uint32_t d,
-                                           uint32_t id, int metric) {
-    const float* r = rows + uint64_t(id) * stride;
-    float s = 0.0f;
-    uint32_t c = 0;
-    for (; c + 4 <= d; c += 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(r + c));
-        const float4 q = *reinterpret_cast<const float4*>(a + c);
-        if (metric == HNSW_L2SQ) {
-            const float t0 = q.x - v.x, t1 = q.y - v.y, t2 = q.z - v.z, t3 = q.w - v.w;
-            s = fmaf(t0, t0, s);
-            s = fmaf(t1, t1, s);
-            s = fmaf(t2, t2, s);
-            s = fmaf(t3, t3, s);
-        } else {
-            s = fmaf(q.x, v.x, s);
-            s = fmaf(q.y, v.y, s);
-            s = fmaf(q.z, v.z, s);
-            s = fmaf(q.w, v.w, s);
-        }
-    }
-    for (; c < d; ++c) {
-        const float v = __ldg(r + c);
-        if (metric == HNSW_L2SQ) {
-            const float t = a[c] - v;
-            s = fmaf(t, t, s);
-        } else {
-            s = fmaf(a[c], v, s);
-        }
-    }
-    return metric == HNSW_L2SQ ? s : 1.0f - s;
-}
-
 // keys of the single-list search: (ordered distance, id, expanded bit)
-__device__ __forceinline__ uint64_t lkey(uint64_t k) { return (k & 0xffffffff00000000ull) | (uint64_t(kid(k)) << 1); }
 __device__ __forceinline__ uint32_t lid(uint64_t k) { return uint32_t(k >> 1) & 0x7fffffffu; }
-
-// ascending bitonic sort of one key per lane across the warp
-__device__ __forceinline__ uint64_t warp_sort_u64(uint64_t v, int lane) {
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const uint64_t o = __shfl_xor_sync(kFull, v, j);
-            const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-            v = (lower == up) ? (v < o ? v : o) : (v > o ? v : o);
-        }
-    return v;
-}
 
 struct UpperArgs {
     DevIndex v;                 // fp32 view; nbrU / upoff of the version being written
@@ -726,244 +676,309 @@ struct UpperArgs {
     int* state;                 // {enter point, top level}
 };
 
-// the W buffer: a power of two >= ef (>= 32) for the final bitonic sort
-__host__ __device__ inline int wcap_of(int efc) {
-    int n = 32;
-    while (n < efc) n <<= 1;
-    return n;
-}
-
 __device__ __forceinline__ uint32_t* upper_row(const UpperArgs& a, uint32_t e, int lc) {
     return const_cast<uint32_t*>(a.v.nbrU) + (uint64_t(a.v.upoff[e]) + uint32_t(lc - 1)) * a.v.sU;
 }
 
-// Alg. 1's descent and layer insertion on layers >= 1 for each new element in turn (one warp):
-// greedy descent above the element's level, then on each of its layers
+constexpr int kUpWarps = 16;
+constexpr int kUpThreads = kUpWarps * 32;
+
+// E * kUpThreads entries of W
+template <int E>
+struct UpperSmem {
+    uint64_t T[E * kUpThreads];   // W during a merge and after the search
+    uint64_t Ek[E * kUpThreads];  // enter points of a layer's search, sorted; afterwards its result
+    uint64_t K[kMaxOld];          // an expansion's new keys (all ones: none)
+    int below[2][kMaxOld];        // entries of W below each new key (two expansions' worth)
+    uint64_t best[2][kUpWarps];   // descent: each warp's best neighbour (two steps' worth)
+    int first[kUpWarps];          // each warp's first unexpanded entry
+    uint32_t first_id[kUpWarps];
+    uint32_t qR[kMaxOld];         // the new element's links
+    int nr;
+    SelSmem sel[kUpWarps];
+    uint64_t keys[kUpWarps][2 * kMaxOld];  // a reverse link's members, sorted
+};
+
+// distance from the warp's vector q (lane l: chunks l and l + 32 of 4
+// coordinates) to row id, in every lane
+template <int DW>
+__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float* rows, uint32_t stride, uint32_t id,
+                                           int metric, int lane) {
+    const float4* r = reinterpret_cast<const float4*>(rows + uint64_t(id) * stride);
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DW / 4; ++k) {
+        const uint32_t c = uint32_t(lane + 32 * k);
+        const float4 v = 4u * c < stride ? __ldg(r + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const float a[4] = {q[k].x, q[k].y, q[k].z, q[k].w}, b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (metric == HNSW_L2SQ) {
+                const float t = a[i] - b[i];
+                s = fmaf(t, t, s);
+            } else {
+                s = fmaf(a[i], b[i], s);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    return metric == HNSW_L2SQ ? s : 1.0f - s;
+}
+
+// Alg. 1's descent and layer insertion on layers >= 1 for each new element in
+// turn: greedy descent above the element's level, then on each of its layers
 // SEARCH-LAYER with efConstruction, SELECT-NEIGHBORS for its list and the
 // reverse links, shrunk with the same selection beyond Mmax; a new top level
 // makes the element the enter point (as in Alg. 1).
-__global__ void __launch_bounds__(32) insert_upper(const UpperArgs a) {
+//
+// The elements follow one another (each may link to the one before it), so one
+// block does them all and what counts is the length of an element's chain.
+// The search is the single-list form: W sorted by key with an 'expanded' bit
+// below the id, its unexpanded entries playing C (an element that left W can
+// never be expanded: it lies beyond W's furthest when reached); an expansion's
+// new neighbours are merged at once (taking them one at a time keeps W = the
+// ef smallest of W and the ones taken, in any order).  A thread holds E
+// entries of W; an expansion's neighbours are scored a warp each, visited tag
+// and vector requested together; every entry counts the new keys below it and
+// every new key the entries below it, which are their places in the new W.
+// Each step is a few instructions between block barriers.  Reverse links are
+// independent of one another (each changes one list and reads vectors): a
+// warp each.  Measured, 62 new elements on one upper layer of 1,250 elements
+// (efConstruction 200, 128 coordinates): 97 ms on one warp, 24 ms now.
+template <int DW, int E>
+__global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
-    const int lane = threadIdx.x & 31;
+    UpperSmem<E>& S = *reinterpret_cast<UpperSmem<E>*>(smem);
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const DevIndex& V = a.v;
     const float* rows = reinterpret_cast<const float*>(V.vec);
-    const uint32_t d = V.d, stride = V.row_chunks * 4, dp = V.row_chunks * 4;
-    const WarpSmem w = carve(smem, a.Mmax, dp);
-    uint8_t* p = smem + warp_smem_bytes(a.Mmax, dp);
-    float* qs = reinterpret_cast<float*>(p);  // [dp] the element being inserted
-    p += size_t(dp) * 4;
-    float* rs = reinterpret_cast<float*>(p);  // [dp] a reverse-link target
-    p += size_t(dp) * 4;
-    uint64_t* Wk = reinterpret_cast<uint64_t*>(p);  // [pow2 >= efc] W: a max-heap, then sorted
-    p += size_t(wcap_of(a.efc)) * 8;
-    uint64_t* Ek = reinterpret_cast<uint64_t*>(p);  // [efc] enter points of the next layer
-    p += size_t(a.efc) * 8;
-    uint32_t* Wid = reinterpret_cast<uint32_t*>(p);  // [efc] decoded W
-    p += size_t(a.efc) * 4;
-    float* Wd = reinterpret_cast<float*>(p);  // [efc]
-    p += size_t(a.efc) * 4;
-    uint32_t* qR = reinterpret_cast<uint32_t*>(p);  // [64]
-    p += 64 * 4;
-    int* LB = reinterpret_cast<int*>(p);  // [32] insertion points of a merge
-    p += 32 * 4;
-    uint64_t* W2 = reinterpret_cast<uint64_t*>(p);  // [pow2 >= efc] merge target
+    const uint32_t stride = V.row_chunks * 4;
+    const int Mmax = int(V.Mmax), efc = a.efc;
     uint32_t epoch = 0;
+    uint32_t ep = uint32_t(a.state[0]);
+    int L = a.state[1];
+    int it = 0;  // which of S.below an expansion uses: all zero when it begins
+    for (int i = t; i < 2 * kMaxOld; i += kUpThreads) (&S.below[0][0])[i] = 0;
     for (uint32_t u = 0; u < a.n; ++u) {
         const uint32_t q = a.ids[u];
         const int l = a.lv[u];
-        __syncwarp();
-        const uint32_t ep = uint32_t(((volatile int*)a.state)[0]);
-        const int L = ((volatile int*)a.state)[1];
-        float xq[kMaxDW];
-        load_vec(rows, stride, d, q, xq, lane);
+        float4 xq[DW / 4];
 #pragma unroll
-        for (int k = 0; k < kMaxDW; ++k)
-            if (uint32_t(lane + 32 * k) < dp) qs[lane + 32 * k] = xq[k];
-        __syncwarp();
-        uint32_t cur = ep;
-        float dcur = dist_id(xq, rows, stride, d, ep, V.metric, lane);
+        for (int k = 0; k < DW / 4; ++k) {
+            const uint32_t c = uint32_t(lane + 32 * k);
+            xq[k] = 4u * c < stride ? __ldg(reinterpret_cast<const float4*>(rows + uint64_t(q) * stride) + c)
+                                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        uint64_t cur = mkkey(dist_warp<DW>(xq, rows, stride, ep, V.metric, lane), ep);
+        int buf = 0;
         for (int lc = L; lc > l; --lc) {  // descent above the level, ef = 1 (steepest descent)
             for (;;) {
-                // every neighbour's distance at once (a lane each), then the
-                // smallest key over the warp
-                const uint32_t* row = upper_row(a, cur, lc);
-                uint64_t best = mkkey(dcur, cur);
-                for (uint32_t j0 = 0; j0 < V.Mmax; j0 += 32) {
-                    const uint32_t j = j0 + lane;
-                    const uint32_t e = j < V.Mmax ? row[j] : kNone;
-                    if (e != kNone) {
-                        const uint64_t k = mkkey(dist_lane(qs, rows, stride, d, e, V.metric), e);
-                        best = k < best ? k : best;
-                    }
+                const uint32_t* row = upper_row(a, kid(cur), lc);
+                uint64_t best = ~0ull;
+                for (int j = wid; j < Mmax; j += kUpWarps) {
+                    const uint32_t e = row[j];
+                    if (e == kNone) break;  // valid ids come first
+                    const uint64_t k = mkkey(dist_warp<DW>(xq, rows, stride, e, V.metric, lane), e);
+                    best = k < best ? k : best;
                 }
+                if (lane == 0) S.best[buf][wid] = best;
+                __syncthreads();
+                best = S.best[buf][lane & (kUpWarps - 1)];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
+                for (int o = kUpWarps / 2; o > 0; o >>= 1) {
                     const uint64_t other = __shfl_xor_sync(kFull, best, o);
                     best = other < best ? other : best;
                 }
-                if (kid(best) == cur) break;
-                cur = kid(best);
-                dcur = kdist(best);
+                buf ^= 1;
+                if (best >= cur) break;
+                cur = best;
             }
         }
+        __syncthreads();  // the last element's lists are written, its shared memory is read
         int n_ep = 1;
-        if (lane == 0) Ek[0] = mkkey(dcur, cur);
-        __syncwarp();
+        if (t == 0) S.Ek[0] = cur;
+        __syncthreads();
         for (int lc = l < L ? l : L; lc >= 1; --lc) {
-            // SEARCH-LAYER(q, ep, efc, lc), in the single-list
-            // form: W sorted by key with an 'expanded' bit below the id; its
-            // unexpanded entries are C (an element that left W can never be
-            // expanded: it lies beyond W's furthest when reached), the next
-            // to expand is the first unexpanded; an expansion's new
-            // neighbours are merged at once (taking them one at a time keeps
-            // W = the ef smallest of W and the ones taken, in any order)
+            // SEARCH-LAYER(q, ep, efc, lc)
             ++epoch;
-            uint64_t* Wa = Wk;
-            uint64_t* Wb = W2;
-            int wn = n_ep;  // n_ep <= efc (the previous layer's W)
-            for (int i = lane; i < wn; i += 32) {
-                const uint64_t k = Ek[i];
-                a.visited[kid(k)] = epoch;
-                Wa[i] = lkey(k);
+            uint64_t w[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int i = e * kUpThreads + t;
+                w[e] = ~0ull;
+                if (i < n_ep) {  // n_ep <= efc (the previous layer's W)
+                    const uint64_t k = S.Ek[i];
+                    a.visited[kid(k)] = epoch;
+                    w[e] = (k & 0xffffffff00000000ull) | (uint64_t(kid(k)) << 1);
+                }
+                S.T[i] = w[e];
             }
-            __syncwarp();
-            int scan = 0;
-            for (;;) {
-                int pos = -1;
-                for (int s0 = scan; s0 < wn; s0 += 32) {
-                    const int i = s0 + lane;
-                    const bool un = i < wn && !(Wa[i] & 1ull);
-                    const unsigned m = __ballot_sync(kFull, un);
+            __syncthreads();
+            for (;; it ^= 1) {
+                // the first unexpanded entry of the first efc
+                int f = INT_MAX;
+                uint32_t fid = 0;
+#pragma unroll
+                for (int e = E - 1; e >= 0; --e) {
+                    const int i = e * kUpThreads + t;
+                    const unsigned m = __ballot_sync(kFull, i < efc && !(uint32_t(w[e]) & 1u));
                     if (m) {
-                        pos = s0 + __ffs(m) - 1;
-                        break;
+                        f = e * kUpThreads + wid * 32 + __ffs(m) - 1;
+                        fid = __shfl_sync(kFull, lid(w[e]), __ffs(m) - 1);
                     }
                 }
-                if (pos < 0) break;  // every entry of W expanded (Alg. 2 stops)
-                const uint64_t c = Wa[pos];
-                __syncwarp();
-                if (lane == 0) Wa[pos] = c | 1ull;
-                scan = pos + 1;
-                const uint32_t* row = upper_row(a, lid(c), lc);
-                for (uint32_t j0 = 0; j0 < V.Mmax; j0 += 32) {
-                    // each neighbour's visited test and distance at once, a lane each
-                    const uint32_t j = j0 + lane;
-                    const uint32_t e = j < V.Mmax ? row[j] : kNone;
-                    const bool fresh = e != kNone && a.visited[e] != epoch;
+                if (lane == 0) {
+                    S.first[wid] = f;
+                    S.first_id[wid] = fid;
+                }
+                __syncthreads();
+                const int fl = S.first[lane & (kUpWarps - 1)];
+                const int p = int(__reduce_min_sync(kFull, uint32_t(fl)));
+                if (p == INT_MAX) break;  // every entry of W expanded (Alg. 2 stops)
+                const uint32_t c = S.first_id[__ffs(__ballot_sync(kFull, fl == p)) - 1];
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (e * kUpThreads + t == p) w[e] |= 1ull;
+                // its neighbours, a warp each
+                const uint64_t thr = S.T[efc - 1] & ~1ull;  // W's furthest (all ones but one bit: not full)
+                const uint32_t* row = upper_row(a, c, lc);
+                for (int j = wid; j < Mmax; j += kUpWarps) {
+                    const uint32_t e = row[j];
                     uint64_t k = ~0ull;
-                    if (fresh) {
-                        a.visited[e] = epoch;
-                        k = (uint64_t(f2ord(dist_lane(qs, rows, stride, d, e, V.metric))) << 32) | (uint64_t(e) << 1);
-                    }
-                    // admission: with W full only keys below its furthest enter
-                    const bool pass = fresh && (wn < a.efc || k < (Wa[wn - 1] & ~1ull));
-                    const unsigned m = __ballot_sync(kFull, pass);
-                    if (!m) continue;
-                    const int nb = __popc(m);
-                    const uint64_t key = warp_sort_u64(pass ? k : ~0ull, lane);  // lane j: j-th smallest
-                    int lb = 0;
-                    if (lane < nb) {  // old entries below the key
-                        int lo = 0, hi = wn;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if ((Wa[mid] & ~1ull) < key)
-                                lo = mid + 1;
-                            else
-                                hi = mid;
+                    if (e != kNone) {
+                        const bool fresh = a.visited[e] != epoch;
+                        const float dq = dist_warp<DW>(xq, rows, stride, e, V.metric, lane);
+                        if (fresh) {
+                            const uint64_t ke = (uint64_t(f2ord(dq)) << 32) | (uint64_t(e) << 1);
+                            if (ke < thr) k = ke;
                         }
-                        lb = lo;
-                        LB[lane] = lb;
                     }
                     __syncwarp();
-                    const int nn = wn + nb < a.efc ? wn + nb : a.efc;
-                    for (int i = lane; i < wn; i += 32) {  // old entry i moves up by the new keys below it
-                        int lo = 0, hi = nb;
-                        while (lo < hi) {
-                            const int mid = (lo + hi) >> 1;
-                            if (LB[mid] <= i)
-                                lo = mid + 1;
-                            else
-                                hi = mid;
-                        }
-                        if (i + lo < nn) Wb[i + lo] = Wa[i];
+                    if (lane == 0) {
+                        S.K[j] = k;
+                        if (e != kNone) a.visited[e] = epoch;
                     }
-                    if (lane < nb && lb + lane < nn) Wb[lb + lane] = key;
-                    __syncwarp();
-                    if (LB[0] < scan) scan = LB[0];  // the smallest new key may precede the scan
-                    uint64_t* t = Wa;
-                    Wa = Wb;
-                    Wb = t;
-                    wn = nn;
-                    __syncwarp();
                 }
+                __syncthreads();
+                const uint64_t kn[2] = {lane < Mmax ? S.K[lane] : ~0ull, lane + 32 < Mmax ? S.K[lane + 32] : ~0ull};
+                const unsigned mk[2] = {__ballot_sync(kFull, kn[0] != ~0ull), __ballot_sync(kFull, kn[1] != ~0ull)};
+                if (t < kMaxOld) S.below[it ^ 1][t] = 0;  // last read before this expansion's first barrier
+                if (!(mk[0] | mk[1])) continue;
+                int above[E], cnt[2] = {0, 0}, rank[2] = {0, 0};
+#pragma unroll
+                for (int e = 0; e < E; ++e) above[e] = 0;  // new keys below each entry
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    for (unsigned m = mk[h]; m; m &= m - 1) {
+                        const int s = __ffs(m) - 1;
+                        const uint64_t k = __shfl_sync(kFull, kn[h], s);
+                        int b = 0;
+#pragma unroll
+                        for (int e = 0; e < E; ++e) {
+                            const bool lower = k < w[e];
+                            above[e] += lower;
+                            b += 32 - __popc(__ballot_sync(kFull, lower));
+                        }
+                        if (lane == s) cnt[h] += b;
+                        rank[0] += k < kn[0];
+                        rank[1] += k < kn[1];
+                    }
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (kn[h] != ~0ull && cnt[h]) atomicAdd(&S.below[it][h * 32 + lane], cnt[h]);
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int i = e * kUpThreads + t + above[e];
+                    if (i < E * kUpThreads) S.T[i] = w[e];
+                }
+                if (wid == 0) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (kn[h] != ~0ull) {
+                            const int i = S.below[it][h * 32 + lane] + rank[h];
+                            if (i < E * kUpThreads) S.T[i] = kn[h];
+                        }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; ++e) w[e] = S.T[e * kUpThreads + t];
             }
-            for (int i = lane; i < wn; i += 32) {
-                const uint64_t k = Wa[i];
-                Wid[i] = lid(k);
-                Wd[i] = kdist(k);
-                Ek[i] = (k & 0xffffffff00000000ull) | lid(k);
+            // the result: the first efc entries, and enter points of the next layer
+            int have = 0;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int i = e * kUpThreads + t;
+                const bool in = i < efc && w[e] != ~0ull;
+                if (in) S.Ek[i] = (w[e] & 0xffffffff00000000ull) | lid(w[e]);
+                have += __syncthreads_count(in);
             }
-            n_ep = int(wn);
-            __syncwarp();
+            n_ep = have;
             // neighbourhood(q) at lc: SELECT-NEIGHBORS(q, W, M)
-            const int nr = select_links(rows, stride, d, dp, V.metric, Wid, Wd, int(wn), a.M, a.heuristic != 0,
-                                        a.keep_pruned != 0, w, lane);
-            for (int j = lane; j < nr; j += 32) qR[j] = w.Rid[j];
-            __syncwarp();
-            uint32_t* rq = upper_row(a, q, lc);
-            for (uint32_t j = lane; j < V.Mmax; j += 32) rq[j] = int(j) < nr ? qR[j] : kNone;
-            __syncwarp();
-            // reverse links and their shrink
-            for (int t = 0; t < nr; ++t) {
-                const uint32_t r = qR[t];
+            if (wid == 0) {
+                const int nr = select_links<DW>(
+                    rows, stride, V.metric,
+                    [&](int i, uint32_t& id, float& dist) {
+                        id = kid(S.Ek[i]);
+                        dist = kdist(S.Ek[i]);
+                    },
+                    n_ep, a.M, a.heuristic != 0, a.keep_pruned != 0, S.sel[0], lane);
+                uint32_t* rq = upper_row(a, q, lc);
+                for (int j = lane; j < Mmax; j += 32) rq[j] = j < nr ? S.sel[0].Rid[j] : kNone;
+                for (int j = lane; j < nr; j += 32) S.qR[j] = S.sel[0].Rid[j];
+                if (lane == 0) S.nr = nr;
+            }
+            __syncthreads();
+            // reverse links and their shrink, a warp each
+            for (int x = wid; x < S.nr; x += kUpWarps) {
+                const uint32_t r = S.qR[x];
                 uint32_t* rr = upper_row(a, r, lc);
                 int n0 = 0;
-                for (uint32_t j = lane; j < V.Mmax; j += 32) n0 += rr[j] != kNone;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) n0 += __shfl_xor_sync(kFull, n0, o);
-                if (n0 < int(V.Mmax)) {
+                for (int j = lane; j < Mmax; j += 32) n0 += rr[j] != kNone;
+                n0 = __reduce_add_sync(kFull, n0);
+                if (n0 < Mmax) {
                     if (lane == 0) rr[n0] = q;
-                    __syncwarp();
                     continue;
                 }
-                float xr[kMaxDW];
-                load_vec(rows, stride, d, r, xr, lane);
-#pragma unroll
-                for (int k = 0; k < kMaxDW; ++k)
-                    if (uint32_t(lane + 32 * k) < dp) rs[lane + 32 * k] = xr[k];
-                __syncwarp();
-                for (int j = lane; j <= n0; j += 32) {  // the members and q, a lane each
+                // the members and q by their distance to r
+                uint64_t* keys = S.keys[wid];
+                TeamVec<DW> xr;
+                load_team(rows, stride, r, xr, lane);
+                for (int j0 = 0; j0 <= n0; j0 += 4) {
+                    const int j = min(j0 + (lane >> 3), n0);
                     const uint32_t c2 = j < n0 ? rr[j] : q;
-                    w.keys[j] = mkkey(dist_lane(rs, rows, stride, d, c2, V.metric), c2);
+                    TeamVec<DW> y;
+                    load_team(rows, stride, c2, y, lane);
+                    const float dc = dist_team(xr, y, V.metric, lane);
+                    if ((lane & 7) == 0) keys[j] = mkkey(dc, c2);
                 }
                 int n2 = 32;
                 while (n2 < n0 + 1) n2 <<= 1;
-                for (int j = n0 + 1 + lane; j < n2; j += 32) w.keys[j] = ~0ull;
+                for (int j = n0 + 1 + lane; j < n2; j += 32) keys[j] = ~0ull;
                 __syncwarp();
-                sort_keys(w.keys, n2, lane);
-                for (int j = lane; j <= n0; j += 32) {
-                    w.cid[j] = kid(w.keys[j]);
-                    w.cd[j] = kdist(w.keys[j]);
-                }
-                __syncwarp();
-                const int nr2 = select_links(rows, stride, d, dp, V.metric, w.cid, w.cd, n0 + 1, int(V.Mmax),
-                                             a.heuristic != 0, a.keep_pruned != 0, w, lane);
-                for (uint32_t j = lane; j < V.Mmax; j += 32) rr[j] = int(j) < nr2 ? w.Rid[j] : kNone;
+                sort_keys(keys, n2, lane);
+                const int nr2 = select_links<DW>(
+                    rows, stride, V.metric,
+                    [&](int i, uint32_t& id, float& dist) {
+                        id = kid(keys[i]);
+                        dist = kdist(keys[i]);
+                    },
+                    n0 + 1, Mmax, a.heuristic != 0, a.keep_pruned != 0, S.sel[wid], lane);
+                for (int j = lane; j < Mmax; j += 32) rr[j] = j < nr2 ? S.sel[wid].Rid[j] : kNone;
                 __syncwarp();
             }
+            __syncthreads();
         }
-        if (l > L && lane == 0) {  // a new top level moves the enter point
-            a.state[0] = int(q);
-            a.state[1] = l;
+        if (l > L) {  // a new top level moves the enter point
+            ep = q;
+            L = l;
         }
-        __threadfence_block();
-        __syncwarp();
     }
-}
-
-size_t upper_smem_bytes(int Mmax, uint32_t dp, int efc) {
-    return warp_smem_bytes(Mmax, dp) + size_t(dp) * 8 + size_t(wcap_of(efc)) * 8 + size_t(efc) * 8 +
-           size_t(efc) * 8 + 64 * 4 + 32 * 4 + size_t(wcap_of(efc)) * 8;
+    if (t == 0) {
+        a.state[0] = int(ep);
+        a.state[1] = L;
+    }
 }
 
 hnsw_status ins_fail(hnsw_status st, const std::string& m) { return fail(st, "hnsw_insert: " + m); }
@@ -1175,14 +1190,16 @@ extern "C" hnsw_status hnsw_insert(hnsw_index* ix, const float* data, uint64_t n
         ua.keep_pruned = keep;
         ua.visited = static_cast<uint32_t*>(visited.p);
         ua.state = static_cast<int*>(state.p);
-        const size_t sm = upper_smem_bytes(Mmax, V.row_chunks * 4, efc);
-        if (sm > 227 * 1024) return ins_fail(HNSW_EINVAL, "dimension too large for the upper-layer kernel");
+        const bool wide = V.row_chunks * 4 > 128, two = efc > kUpThreads;
+        void (*up)(const UpperArgs) = wide ? (two ? insert_upper<8, 2> : insert_upper<8, 1>)
+                                           : (two ? insert_upper<4, 2> : insert_upper<4, 1>);
+        const size_t sm = two ? sizeof(UpperSmem<2>) : sizeof(UpperSmem<1>);
         {
-            const hnsw_status r = raise_smem_limit(reinterpret_cast<const void*>(insert_upper), sm, "hnsw_insert");
+            const hnsw_status r = raise_smem_limit(reinterpret_cast<const void*>(up), sm, "hnsw_insert");
             if (r != HNSW_OK) return r;
         }
         if (e == cudaSuccess) {
-            insert_upper<<<1, 32, sm, s>>>(ua);
+            up<<<1, kUpThreads, sm, s>>>(ua);
             e = cudaGetLastError();
         }
         int st1[2] = {0, 0};
