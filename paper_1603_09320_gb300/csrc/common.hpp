@@ -33,9 +33,9 @@ struct BlobLayout {
     }
 };
 
-// 64-bit FNV-1a over a byte range, 8 bytes per step of the outer loop.
-inline uint64_t fnv1a64(const uint8_t* p, uint64_t n) {
-    uint64_t h = 0xcbf29ce484222325ull;
+// 64-bit FNV-1a over a byte range (going on from h).
+constexpr uint64_t kFnvBasis = 0xcbf29ce484222325ull;
+inline uint64_t fnv1a64(const uint8_t* p, uint64_t n, uint64_t h = kFnvBasis) {
     const uint64_t prime = 0x100000001b3ull;
     for (uint64_t i = 0; i < n; ++i) {
         h ^= p[i];
@@ -101,11 +101,16 @@ inline bool read_header(const uint8_t* b, uint64_t bytes, BlobHeader& h) {
     return h.version == 1;
 }
 
+// A checksum of n bytes at p (ctx: the caller's).
+using ChecksumFn = uint64_t (*)(const uint8_t* p, uint64_t n, void* ctx);
+
 // Full structural validation of a blob; on success fills `h`, the layout and
 // the per-element first-upper-row offsets (kNoId for level-0 elements).
 // full = false (a blob the library has just written itself): header, sizes
-// and offsets only -- no checksum, no per-list checks.
+// and offsets only -- no checksum, no per-list checks.  sum: computes the
+// checksum (null: fnv1a64).
 hnsw_status validate_blob(const uint8_t* b, uint64_t bytes, BlobHeader& h, BlobLayout& lay,
-                          std::vector<uint32_t>& upoff, bool full = true);
+                          std::vector<uint32_t>& upoff, bool full = true, ChecksumFn sum = nullptr,
+                          void* ctx = nullptr);
 
 }  // namespace hnswgb

@@ -613,7 +613,7 @@ extern "C" hnsw_status hnsw_build_gpu(const float* data, uint64_t N, uint32_t d,
     h.n_upper_rows = rows;
     hnsw_free_blob(sblob);
     auto finish_header = [&]() {
-        h.checksum = fnv1a64(b + 128, lay.total - 128);
+        h.checksum = checksum64(b + 128, lay.total - 128, s);
         write_header(b, h);
     };
     // 2. layer-0 insertion of the rest on the GPU (the intermediate blob is
@@ -1277,7 +1277,7 @@ extern "C" hnsw_status hnsw_index_to_blob(hnsw_index* ix, void** out_blob, uint6
     h.efC = ix->build_efC;
     h.mL = ix->build_mL;
     h.n_upper_rows = ix->upper_rows;
-    h.checksum = fnv1a64(b + 128, lay.total - 128);
+    h.checksum = checksum64(b + 128, lay.total - 128, nullptr);
     write_header(b, h);
     *out_blob = b;
     *out_bytes = lay.total;

@@ -101,7 +101,9 @@ hnsw_status upload_index(const void* graph_blob, uint64_t blob_bytes, hnsw_dtype
     BlobHeader h{};
     BlobLayout lay{};
     std::vector<uint32_t> upoff;
-    hnsw_status st = validate_blob(b, blob_bytes, h, lay, upoff, !trusted);
+    hnsw_status st = validate_blob(
+        b, blob_bytes, h, lay, upoff, !trusted,
+        [](const uint8_t* p, uint64_t n, void* s) { return checksum64(p, n, static_cast<cudaStream_t>(s)); }, stream);
     if (st != HNSW_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const uint64_t N = h.N;
