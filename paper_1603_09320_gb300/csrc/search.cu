@@ -264,11 +264,18 @@ enum class Defer { no, automatic, always };
 // per query.  The block kernel shortens a query's chain but spends more
 // instructions and registers on it, so it is taken while all queries of the
 // batch are resident at once: up to two 8-warp blocks per SM, then up to four
-// 4-warp blocks (both sides of the limits: search_team.cuh).
+// 4-warp blocks (both sides of the limits: search_team.cuh).  Beams above 256
+// keep more of W in registers and shared memory: three 4-warp blocks (ef 498,
+// warp per query / block: 400 queries 1.24 times the time, 608 on GloVe-shaped
+// data 0.83 to 0.88 times).  Rows of up to 32 bytes leave little to score
+// ahead: with beams above 64 and no rerank a warp per query is as quick or
+// quicker (8 fp32 coordinates, ef 200, 8 to 60 queries: 0.86 to 0.96 times).
 int team_warps(const DevIndex& D, const hnsw_search_params& p, uint32_t n) {
-    if (p.schedule != 0 || p.check_bounds || D.N == 0 || D.N >= kTeamMaxN || std::max(p.ef, p.k) > 512) return 0;
+    const int efp = std::max(p.ef, p.k);
+    if (p.schedule != 0 || p.check_bounds || D.N == 0 || D.N >= kTeamMaxN || efp > 512) return 0;
+    if (D.row_chunks <= 2 && efp > 64 && !p.rerank) return 0;
     const uint32_t sms = uint32_t(sm_count());
-    return n <= 2 * sms ? 8 : n <= 4 * sms ? 4 : 0;
+    return n <= 2 * sms ? 8 : n <= (efp > 256 ? 3 : 4) * sms ? 4 : 0;
 }
 
 // Launches the block-per-query kernel fn with nw warps per block on the
@@ -293,7 +300,7 @@ hnsw_status launch_team(SearchArgs& a, KernelFn fn, int nw, int visited_log2, cu
     };
     const int sms = sm_count();
     auto resident = [&](size_t smem) { return uint64_t(std::max(0, blocks_per_sm(fn, nw * 32, smem))) * sms; };
-    const int most = visited_log2 > 0 ? visited_log2 : std::min(14, std::max(11, ceil_log2(uint64_t(a.efp) * 32)));
+    const int most = visited_log2 > 0 ? visited_log2 : std::min(14, std::max(11, ceil_log2(uint64_t(a.efp) * 64)));
     if (layout(most) > 227 * 1024) return fail(HNSW_EINVAL, "search: ef/visited set too large for shared memory");
     const hnsw_status st = raise_smem_limit(reinterpret_cast<const void*>(fn), layout(most), "search");
     if (st != HNSW_OK) return st;

@@ -570,22 +570,42 @@ __device__ __forceinline__ int merge_small(uint64_t* W, int& size, int efp, uint
     return int(__reduce_min_sync(kFull, uint32_t(pos)));
 }
 
-// W of up to 1,024 entries.  Lower bounds by binary search, ranks among the
+// W of up to 1,024 entries.  Lower bounds by ballots (BALLOT: where registers
+// are left for them) or binary search, ranks among the
 // survivors as above; the final positions of the new keys are then a bitmap
-// (one 32-bit word per lane: 1,024 positions) whose prefix counts say for
-// every other position where its entry comes from, so that W moves up in one
-// pass over its 32-entry chunks, top chunk first, with a few instructions per
-// chunk whatever the number of new keys.  (The form that counted, for every
+// (one 32-bit word per lane: 1,024 positions); the count of its bits below a
+// position says where that position's entry comes from, so that W moves up in
+// one pass over its 32-entry chunks, top chunk first, with a few instructions
+// per chunk whatever the number of new keys.  (The form that counted, for every
 // entry, the new keys placed before it took a pass over the new keys per
-// chunk: GloVe-shaped 400k, 10,000 queries at ef 498: 7.19 ms, 6.03 ms with
+// chunk: GloVe-shaped 400k, 10,000 queries at ef 498: 7.19 ms, 5.85 ms with
 // this merge and the shorter row distances.)
+template <bool BALLOT>
 __device__ __forceinline__ int merge_wide(uint64_t* W, int& size, int efp, uint64_t k, bool& ok, int lane) {
     const uint64_t wlast = size > 0 ? (W[size - 1] >> 1) : 0ull;
     const uint64_t k1 = k >> 1;
     ok = ok && !(size >= efp && k1 > wlast);
-    if (!__any_sync(kFull, ok)) return INT_MAX;
+    const uint32_t cand = __ballot_sync(kFull, ok);
+    if (cand == 0) return INT_MAX;
     int lb = 0;
-    if (ok) {
+    if (BALLOT && __popc(cand) <= HNSW_MERGE_BALLOT_MAX) {
+        // few candidates: the 32 entries that hold the place by a ballot over
+        // the last entries of all 32s, the place by one over these (two reads
+        // of shared memory in a row instead of up to ten)
+        const uint64_t top = 32 * lane < size ? W[min(32 * lane + 31, size - 1)] : ~0ull;
+        for (uint32_t bits = cand; bits; bits &= bits - 1) {
+            const int sl = __ffs(bits) - 1;
+            const uint64_t ks = __shfl_sync(kFull, k, sl);  // expanded bit clear
+            const int base = 32 * __popc(__ballot_sync(kFull, top < ks));
+            const uint64_t v = base + lane < size ? W[base + lane] : ~0ull;
+            const int l = min(base + __popc(__ballot_sync(kFull, v < ks)), size);
+            const bool dup = __any_sync(kFull, (v | 1ull) == (ks | 1ull));  // already in W
+            if (lane == sl) {
+                lb = l;
+                ok = !dup;
+            }
+        }
+    } else if (ok) {
         for (int step = 1 << (31 - __clz(size | 1)); step > 0; step >>= 1)  // entries of W below k1
             if (lb + step <= size && (W[lb + step - 1] >> 1) < k1) lb += step;
         if (lb < size && (W[lb] >> 1) == k1) ok = false;  // already in W
@@ -605,17 +625,12 @@ __device__ __forceinline__ int merge_wide(uint64_t* W, int& size, int efp, uint6
         const int p = __shfl_sync(kFull, pos, __ffs(bits) - 1);
         if ((p >> 5) == lane) word |= 1u << (p & 31);
     }
-    int before = __popc(word);  // new positions below this lane's word, after the scan
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(kFull, before, o);
-        if (lane >= o) before += v;
-    }
-    before -= __popc(word);
+    int below = __popc(in);  // new positions below the chunk
     for (int c = (nsize - 1) >> 5; c >= first >> 5; --c) {
         const uint32_t wc = __shfl_sync(kFull, word, c);
+        below -= __popc(wc);
         const int t = c * 32 + lane;
-        const int src = t - __shfl_sync(kFull, before, c) - __popc(wc & lanemask_lt());
+        const int src = t - below - __popc(wc & lanemask_lt());
         const bool mv = !((wc >> lane) & 1u) && t > first && t < nsize;
         const uint64_t v = mv ? W[src] : 0ull;
         __syncwarp();  // a chunk's reads (at most this chunk's positions) precede its writes

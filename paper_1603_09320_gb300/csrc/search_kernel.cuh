@@ -130,6 +130,9 @@ template <int ST, int TEAM, int CPL, int U, bool FULL, bool STOP, bool WIDE, boo
 __global__ void __launch_bounds__(256) __maxnreg__((search_max_regs<ST, TEAM, CPL, U, FULL, STOP, CHECK>()))
     hnsw_search_kernel(const SearchArgs a) {
     using D = Dist<ST, TEAM, CPL, U, FULL>;
+    // full fp32 rows of 128 coordinates have no registers left for the wide
+    // merge's ballots at 72 (56 bytes of spill, 5% slower at ef 66 to 100)
+    constexpr bool kBallot = search_max_regs<ST, TEAM, CPL, U, FULL, STOP, CHECK>() != 72;
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     uint8_t* wbase = smem + (threadIdx.x >> 5) * a.warp_smem;
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((search_max_regs<ST, TEAM, CP
                         const int j = h + lane;
                         bool ok = j < n;
                         const uint64_t key = ok ? mkkey(dst[j], ids[j]) : 0ull;
-                        first_new = min(first_new, WIDE ? merge_wide(W, size, efq, key, ok, lane)
+                        first_new = min(first_new, WIDE ? merge_wide<kBallot>(W, size, efq, key, ok, lane)
                                                         : merge_small(W, size, efq, key, ok, lane));
                     }
                 }
