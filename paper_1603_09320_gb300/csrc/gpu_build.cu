@@ -686,31 +686,35 @@ constexpr int kUpThreads = kUpWarps * 32;
 // E * kUpThreads entries of W
 template <int E>
 struct UpperSmem {
-    uint64_t T[E * kUpThreads];   // W during a merge and after the search
-    uint64_t Ek[E * kUpThreads];  // enter points of a layer's search, sorted; afterwards its result
-    uint64_t K[kMaxOld];          // an expansion's new keys (all ones: none)
-    int below[2][kMaxOld];        // entries of W below each new key (two expansions' worth)
-    uint64_t best[2][kUpWarps];   // descent: each warp's best neighbour (two steps' worth)
-    int first[kUpWarps];          // each warp's first unexpanded entry
-    uint32_t first_id[kUpWarps];
+    uint64_t T[2][E * kUpThreads];  // W, and the W that the next merge makes
+    uint64_t Ek[E * kUpThreads];    // enter points of a layer's search, sorted; afterwards its result
+    uint64_t K[2][kMaxOld];         // an expansion's new keys (all ones: none), two expansions' worth
+    uint32_t ids[2][kMaxOld];       // and its neighbours
+    uint64_t best[2][kUpWarps];     // descent: each warp's best neighbour (two steps' worth)
+    int first;                      // where the smallest new key went
     uint32_t qR[kMaxOld];         // the new element's links
     int nr;
     SelSmem sel[kUpWarps];
     uint64_t keys[kUpWarps][2 * kMaxOld];  // a reverse link's members, sorted
 };
 
-// distance from the warp's vector q (lane l: chunks l and l + 32 of 4
-// coordinates) to row id, in every lane
+// A row in the registers of a warp (lane l: chunks l and l + 32 of 4 coordinates).
 template <int DW>
-__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float* rows, uint32_t stride, uint32_t id,
-                                           int metric, int lane) {
+__device__ __forceinline__ void load_warp(float4 (&v)[DW / 4], const float* rows, uint32_t stride, uint32_t id, int lane) {
     const float4* r = reinterpret_cast<const float4*>(rows + uint64_t(id) * stride);
-    float s = 0.0f;
 #pragma unroll
     for (int k = 0; k < DW / 4; ++k) {
         const uint32_t c = uint32_t(lane + 32 * k);
-        const float4 v = 4u * c < stride ? __ldg(r + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        const float a[4] = {q[k].x, q[k].y, q[k].z, q[k].w}, b[4] = {v.x, v.y, v.z, v.w};
+        v[k] = 4u * c < stride ? __ldg(r + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+}
+// distance between two such rows, in every lane
+template <int DW>
+__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float4 (&v)[DW / 4], int metric) {
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DW / 4; ++k) {
+        const float a[4] = {q[k].x, q[k].y, q[k].z, q[k].w}, b[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (metric == HNSW_L2SQ) {
@@ -725,6 +729,13 @@ __device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const floa
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
     return metric == HNSW_L2SQ ? s : 1.0f - s;
 }
+template <int DW>
+__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float* rows, uint32_t stride, uint32_t id,
+                                           int metric, int lane) {
+    float4 v[DW / 4];
+    load_warp<DW>(v, rows, stride, id, lane);
+    return dist_warp<DW>(q, v, metric);
+}
 
 // Alg. 1's descent and layer insertion on layers >= 1 for each new element in
 // turn: greedy descent above the element's level, then on each of its layers
@@ -738,15 +749,29 @@ __device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const floa
 // below the id, its unexpanded entries playing C (an element that left W can
 // never be expanded: it lies beyond W's furthest when reached); an expansion's
 // new neighbours are merged at once (taking them one at a time keeps W = the
-// ef smallest of W and the ones taken, in any order).  A thread holds E
-// entries of W; an expansion's neighbours are scored a warp each, visited tag
-// and vector requested together; every entry counts the new keys below it and
-// every new key the entries below it, which are their places in the new W.
-// Each step is a few instructions between block barriers.  Reverse links are
-// independent of one another (each changes one list and reads vectors): a
-// warp each.  Measured, 62 new elements on one upper layer of 1,250 elements
-// (efConstruction 200, 128 coordinates): 97 ms on one warp, 24 ms now.
-template <int DW, int E>
+// ef smallest of W and the ones taken, in any order).  W lies in shared memory
+// and, E entries per thread, in registers.  An expansion is
+//  * every warp by itself finds the first unexpanded entry, from `scan` on;
+//  * its neighbours are scored, up to NB by a warp.  The entry after it is
+//    expanded next unless a nearer one turns up, so that one's neighbours,
+//    vectors and visited tags are requested before the scoring is waited for
+//    (a tag read that early misses the neighbours of the expansion in between:
+//    they are compared with);
+//  * each warp that holds entries looks the new keys' places in W up by binary
+//    search; from them follow how far its entries move and, in the first warp,
+//    where the keys go, all into the other copy of W.
+// That is one block barrier, two where something entered W.
+// Reverse links are independent of one another (each changes one list and
+// reads vectors): a warp each.  Measured, 1,000 elements into 20,000, of which 70
+// go to a layer of 1,250 (efConstruction 200, 128 coordinates): the whole
+// insertion call took 99 ms with one warp here, 25.6 with a block that merged
+// by counting, atomics and four barriers an expansion, and takes 24.4.  What
+// bounds it is an expansion's instructions, which follow one another (2,700
+// cycles: 600 to find the entry, 600 to score, 400 for the requests, 2,000
+// where keys are merged, which is every other time), not the reads.  Slower or
+// the same: 8 warps with a team of 8 lanes per row (25.8 ms), visited elements
+// as a bitmap in shared memory (24.9), vectors read past L1.
+template <int DW, int E, int NB>
 __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     UpperSmem<E>& S = *reinterpret_cast<UpperSmem<E>*>(smem);
@@ -758,8 +783,8 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
     uint32_t epoch = 0;
     uint32_t ep = uint32_t(a.state[0]);
     int L = a.state[1];
-    int it = 0;  // which of S.below an expansion uses: all zero when it begins
-    for (int i = t; i < 2 * kMaxOld; i += kUpThreads) (&S.below[0][0])[i] = 0;
+    int kb = 0;  // which of S.K and S.ids an expansion uses
+    for (int i = t; i < 2 * kMaxOld; i += kUpThreads) (&S.K[0][0])[i] = ~0ull;  // stay so from Mmax on
     for (uint32_t u = 0; u < a.n; ++u) {
         const uint32_t q = a.ids[u];
         const int l = a.lv[u];
@@ -812,98 +837,146 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
                     a.visited[kid(k)] = epoch;
                     w[e] = (k & 0xffffffff00000000ull) | (uint64_t(kid(k)) << 1);
                 }
-                S.T[i] = w[e];
+                S.T[0][i] = w[e];
             }
-            __syncthreads();
-            for (;; it ^= 1) {
-                // the first unexpanded entry of the first efc
-                int f = INT_MAX;
-                uint32_t fid = 0;
+            int cw = 0;              // which of S.T is W
+            int scan = 0;            // the entries before it are expanded
+            uint32_t ahead = kNone;  // the element whose neighbours these are:
+            uint32_t ne[NB], tag[NB];
+            float4 nv[NB][DW / 4];
+            auto request = [&](uint32_t c, uint32_t first_row) {
+                ahead = c;
+                const uint32_t* row = V.nbrU + (uint64_t(first_row) + uint32_t(lc - 1)) * V.sU;
 #pragma unroll
-                for (int e = E - 1; e >= 0; --e) {
-                    const int i = e * kUpThreads + t;
-                    const unsigned m = __ballot_sync(kFull, i < efc && !(uint32_t(w[e]) & 1u));
-                    if (m) {
-                        f = e * kUpThreads + wid * 32 + __ffs(m) - 1;
-                        fid = __shfl_sync(kFull, lid(w[e]), __ffs(m) - 1);
+                for (int k = 0; k < NB; ++k) ne[k] = wid + k * kUpWarps < Mmax ? row[wid + k * kUpWarps] : kNone;
+#pragma unroll
+                for (int k = 0; k < NB; ++k)
+                    if (ne[k] != kNone) {
+                        tag[k] = a.visited[ne[k]];
+                        load_warp<DW>(nv[k], rows, stride, ne[k], lane);
                     }
+            };
+            __syncthreads();
+            for (;; kb ^= 1) {
+                const uint64_t* T = S.T[cw];
+                // the first unexpanded entry, and the one after it
+                int p = -1;
+                uint32_t c = kNone, c2 = kNone;
+                for (int s0 = scan; s0 < efc; s0 += 32) {
+                    const uint32_t lo = s0 + lane < efc ? uint32_t(T[s0 + lane]) : 1u;
+                    unsigned m = __ballot_sync(kFull, !(lo & 1u));
+                    if (!m && p >= 0) break;  // one more window at most for the second
+                    if (m && p < 0) {
+                        const int at = __ffs(m) - 1;
+                        p = s0 + at;
+                        c = __shfl_sync(kFull, lo >> 1, at);
+                        m &= m - 1;
+                    }
+                    if (!m) continue;
+                    c2 = __shfl_sync(kFull, lo >> 1, __ffs(m) - 1);
+                    break;
                 }
-                if (lane == 0) {
-                    S.first[wid] = f;
-                    S.first_id[wid] = fid;
-                }
-                __syncthreads();
-                const int fl = S.first[lane & (kUpWarps - 1)];
-                const int p = int(__reduce_min_sync(kFull, uint32_t(fl)));
-                if (p == INT_MAX) break;  // every entry of W expanded (Alg. 2 stops)
-                const uint32_t c = S.first_id[__ffs(__ballot_sync(kFull, fl == p)) - 1];
+                if (p < 0) break;  // every entry of W expanded (Alg. 2 stops)
 #pragma unroll
                 for (int e = 0; e < E; ++e)
                     if (e * kUpThreads + t == p) w[e] |= 1ull;
-                // its neighbours, a warp each
-                const uint64_t thr = S.T[efc - 1] & ~1ull;  // W's furthest (all ones but one bit: not full)
-                const uint32_t* row = upper_row(a, c, lc);
-                for (int j = wid; j < Mmax; j += kUpWarps) {
-                    const uint32_t e = row[j];
-                    uint64_t k = ~0ull;
+                // its neighbours
+                const uint64_t thr = T[efc - 1] & ~1ull;  // W's furthest (all ones but one bit: not full)
+                const uint32_t row2 = c2 != kNone ? V.upoff[c2] : 0u;
+                const bool early = c == ahead;
+                if (!early) request(c, V.upoff[c]);
+                const uint32_t o0 = early && lane < Mmax ? S.ids[kb ^ 1][lane] : kNone;
+                const uint32_t o1 = early && lane + 32 < Mmax ? S.ids[kb ^ 1][lane + 32] : kNone;
+#pragma unroll
+                for (int k = 0; k < NB; ++k) {
+                    const int j = wid + k * kUpWarps;
+                    if (j >= Mmax) break;
+                    uint64_t key = ~0ull;
+                    const uint32_t e = ne[k];
                     if (e != kNone) {
-                        const bool fresh = a.visited[e] != epoch;
-                        const float dq = dist_warp<DW>(xq, rows, stride, e, V.metric, lane);
-                        if (fresh) {
+                        const float dq = dist_warp<DW>(xq, nv[k], V.metric);
+                        const bool met = __any_sync(kFull, tag[k] == epoch || o0 == e || o1 == e);
+                        if (!met) {
                             const uint64_t ke = (uint64_t(f2ord(dq)) << 32) | (uint64_t(e) << 1);
-                            if (ke < thr) k = ke;
+                            if (ke < thr) key = ke;
                         }
                     }
-                    __syncwarp();
                     if (lane == 0) {
-                        S.K[j] = k;
+                        S.K[kb][j] = key;
+                        S.ids[kb][j] = e;
                         if (e != kNone) a.visited[e] = epoch;
                     }
                 }
+                if (c2 != kNone) request(c2, row2);
                 __syncthreads();
-                const uint64_t kn[2] = {lane < Mmax ? S.K[lane] : ~0ull, lane + 32 < Mmax ? S.K[lane + 32] : ~0ull};
+                const uint64_t kn[2] = {S.K[kb][lane], Mmax > 32 ? S.K[kb][lane + 32] : ~0ull};
                 const unsigned mk[2] = {__ballot_sync(kFull, kn[0] != ~0ull), __ballot_sync(kFull, kn[1] != ~0ull)};
-                if (t < kMaxOld) S.below[it ^ 1][t] = 0;  // last read before this expansion's first barrier
-                if (!(mk[0] | mk[1])) continue;
-                int above[E], cnt[2] = {0, 0}, rank[2] = {0, 0};
+                if (!(mk[0] | mk[1])) {
+                    // entries before `scan` are not looked at until a merge
 #pragma unroll
-                for (int e = 0; e < E; ++e) above[e] = 0;  // new keys below each entry
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    for (unsigned m = mk[h]; m; m &= m - 1) {
-                        const int s = __ffs(m) - 1;
-                        const uint64_t k = __shfl_sync(kFull, kn[h], s);
-                        int b = 0;
-#pragma unroll
-                        for (int e = 0; e < E; ++e) {
-                            const bool lower = k < w[e];
-                            above[e] += lower;
-                            b += 32 - __popc(__ballot_sync(kFull, lower));
-                        }
-                        if (lane == s) cnt[h] += b;
-                        rank[0] += k < kn[0];
-                        rank[1] += k < kn[1];
-                    }
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    if (kn[h] != ~0ull && cnt[h]) atomicAdd(&S.below[it][h * 32 + lane], cnt[h]);
-                __syncthreads();
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const int i = e * kUpThreads + t + above[e];
-                    if (i < E * kUpThreads) S.T[i] = w[e];
+                    for (int e = 0; e < E; ++e)
+                        if (e * kUpThreads + t == p) S.T[cw][p] = w[e];
+                    scan = p + 1;
+                    continue;
                 }
-                if (wid == 0) {
+                uint64_t* T2 = S.T[cw ^ 1];
+                if (wid * 32 < efc) {
+                    int lb[2] = {0, 0}, rank[2] = {0, 0}, above[E];
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
-                        if (kn[h] != ~0ull) {
-                            const int i = S.below[it][h * 32 + lane] + rank[h];
-                            if (i < E * kUpThreads) S.T[i] = kn[h];
+                        if (mk[h])  // entries of W below the key, four ways a step
+                            for (int step = 1 << ((31 - __clz(efc)) & ~1); step > 0; step >>= 2) {
+                                const int b = lb[h] - 1;
+                                int up = 0;
+#pragma unroll
+                                for (int x = 1; x <= 3; ++x)
+                                    up += b + x * step < efc && T[b + x * step] < kn[h];
+                                lb[h] += up * step;
+                            }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if (kn[h] == ~0ull) lb[h] = INT_MAX;  // an empty slot lies below no entry
+#pragma unroll
+                    for (int e = 0; e < E; ++e) above[e] = 0;  // new keys below each entry
+#pragma unroll
+                    for (int g = 0; g < NB; ++g) {  // 16 slots at a time: their reads overlap
+                        if (!(mk[g / 2] >> (16 * (g & 1)) & 0xffffu)) continue;
+#pragma unroll
+                        for (int x = 0; x < 16; ++x) {
+                            const uint64_t k = S.K[kb][16 * g + x];
+                            const int l0 = __shfl_sync(kFull, lb[g / 2], 16 * (g & 1) + x);
+#pragma unroll
+                            for (int e = 0; e < E; ++e) above[e] += l0 <= e * kUpThreads + t;
+                            rank[0] += k < kn[0];
+                            if (NB > 2) rank[1] += k < kn[1];
                         }
+                    }
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int i = e * kUpThreads + t;
+                        if (i < efc && i + above[e] < efc) T2[i + above[e]] = w[e];
+                    }
+                    if (wid == 0) {
+                        int first = INT_MAX;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (kn[h] != ~0ull) {
+                                const int i = lb[h] + rank[h];
+                                if (i < efc) T2[i] = kn[h];
+                                first = min(first, i);
+                            }
+                        first = int(__reduce_min_sync(kFull, uint32_t(first)));
+                        if (lane == 0) S.first = first;
+                    }
                 }
                 __syncthreads();
+                cw ^= 1;
+                scan = min(p + 1, S.first);
 #pragma unroll
-                for (int e = 0; e < E; ++e) w[e] = S.T[e * kUpThreads + t];
+                for (int e = 0; e < E; ++e) {
+                    const int i = e * kUpThreads + t;
+                    w[e] = i < efc ? T2[i] : ~0ull;
+                }
             }
             // the result: the first efc entries, and enter points of the next layer
             int have = 0;
@@ -980,6 +1053,15 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
         a.state[1] = L;
     }
 }
+
+// the instance for lists of up to Mmax (<= kMaxOld)
+template <int DW, int E>
+auto upper_kernel(int Mmax) {
+    return Mmax <= kUpWarps       ? insert_upper<DW, E, 1>
+           : Mmax <= 2 * kUpWarps ? insert_upper<DW, E, 2>
+                                  : insert_upper<DW, E, 4>;
+}
+static_assert(kMaxOld <= 4 * kUpWarps, "a warp scores up to 4 neighbours");
 
 hnsw_status ins_fail(hnsw_status st, const std::string& m) { return fail(st, "hnsw_insert: " + m); }
 
@@ -1191,8 +1273,8 @@ extern "C" hnsw_status hnsw_insert(hnsw_index* ix, const float* data, uint64_t n
         ua.visited = static_cast<uint32_t*>(visited.p);
         ua.state = static_cast<int*>(state.p);
         const bool wide = V.row_chunks * 4 > 128, two = efc > kUpThreads;
-        void (*up)(const UpperArgs) = wide ? (two ? insert_upper<8, 2> : insert_upper<8, 1>)
-                                           : (two ? insert_upper<4, 2> : insert_upper<4, 1>);
+        void (*up)(const UpperArgs) = wide ? (two ? upper_kernel<8, 2>(Mmax) : upper_kernel<8, 1>(Mmax))
+                                           : (two ? upper_kernel<4, 2>(Mmax) : upper_kernel<4, 1>(Mmax));
         const size_t sm = two ? sizeof(UpperSmem<2>) : sizeof(UpperSmem<1>);
         {
             const hnsw_status r = raise_smem_limit(reinterpret_cast<const void*>(up), sm, "hnsw_insert");

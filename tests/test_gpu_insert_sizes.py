@@ -1,6 +1,7 @@
 """Incremental insertion at the edges of its kernels' ranges against the
 oracle's batch form, byte for byte on integer data: selection flags, rows of
-few, ragged and more than 128 coordinates, upper lists of more than 32, a beam
+few, ragged and more than 128 coordinates, upper lists of up to 16, of up to 32
+and of more than 32, a beam
 of more than 512 entries, several upper layers and new top levels."""
 import numpy as np
 import pytest
@@ -15,6 +16,7 @@ SHAPES = [
     (32, 8, 8, 16, 64, 0.8, True, True),
     (5, 6, 7, 13, 33, 0.9, True, False),
     (130, 6, 6, 12, 40, 0.7, True, False),
+    (32, 12, 24, 48, 100, 0.8, True, False),
     (32, 20, 40, 64, 600, 0.6, True, False),
     (32, 20, 40, 64, 600, 0.6, True, True),
 ]
