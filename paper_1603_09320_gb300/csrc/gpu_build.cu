@@ -147,6 +147,7 @@ __device__ int prune(const float* rows, uint32_t stride, int metric, uint32_t r,
     const bool k0 = lane < na && w.keep[lane], k1 = lane + 32 < na && w.keep[lane + 32];
     const uint32_t v0 = k0 ? w.live[lane] : 0u, v1 = k1 ? w.live[lane + 32] : 0u;
     const unsigned m0 = __ballot_sync(kFull, k0), m1 = __ballot_sync(kFull, k1), below = (1u << lane) - 1u;
+    __syncwarp();  // every lane has read its entries before any is overwritten (a ballot orders no memory)
     if (k0) w.live[__popc(m0 & below)] = v0;
     if (k1) w.live[__popc(m0) + __popc(m1 & below)] = v1;
     __syncwarp();
