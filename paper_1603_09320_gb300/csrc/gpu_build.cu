@@ -697,6 +697,8 @@ struct UpperSmem {
     int nr;
     SelSmem sel[kUpWarps];
     uint64_t keys[kUpWarps][2 * kMaxOld];  // a reverse link's members, sorted
+    float4 q[8 * kMaxDW];                  // the new element
+    float4 t[kUpWarps][8 * kMaxDW];        // each warp's row (dist_seq, dist_lane)
 };
 
 // A row in the registers of a warp (lane l: chunks l and l + 32 of 4 coordinates).
@@ -709,33 +711,67 @@ __device__ __forceinline__ void load_warp(float4 (&v)[DW / 4], const float* rows
         v[k] = 4u * c < stride ? __ldg(r + c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 }
-// distance between two such rows, in every lane
+// Distance between q (shared memory, stride floats) and such a row, in every
+// lane, the coordinates added one after another: the order in which the upper
+// layers have always been scored (near-ties decide links).  The warp's lanes
+// hold four coordinates each, so the row goes through t (the warp's shared
+// memory, 8 DW chunks), which every lane then reads from its start.
 template <int DW>
-__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float4 (&v)[DW / 4], int metric) {
-    float s = 0.0f;
+__device__ __forceinline__ float dist_seq(const float4* q, const float4 (&v)[DW / 4], uint32_t stride, int metric,
+                                          float4* t, int lane) {
+    const bool l2 = metric == HNSW_L2SQ;
+    __syncwarp();  // the previous row is read
 #pragma unroll
     for (int k = 0; k < DW / 4; ++k) {
-        const float a[4] = {q[k].x, q[k].y, q[k].z, q[k].w}, b[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (metric == HNSW_L2SQ) {
-                const float t = a[i] - b[i];
-                s = fmaf(t, t, s);
-            } else {
-                s = fmaf(a[i], b[i], s);
-            }
+        const int c = lane + 32 * k;
+        if (4u * c < stride) {
+            const float4 a = q[c];
+            t[c] = l2 ? make_float4(a.x - v[k].x, a.y - v[k].y, a.z - v[k].z, a.w - v[k].w) : v[k];
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    return metric == HNSW_L2SQ ? s : 1.0f - s;
+    __syncwarp();
+    float s = 0.0f;
+    if (l2) {
+#pragma unroll 8
+        for (uint32_t c = 0; 4u * c < stride; ++c) {
+            const float4 a = t[c];
+            s = fmaf(a.x, a.x, s);
+            s = fmaf(a.y, a.y, s);
+            s = fmaf(a.z, a.z, s);
+            s = fmaf(a.w, a.w, s);
+        }
+        return s;
+    }
+#pragma unroll 4
+    for (uint32_t c = 0; 4u * c < stride; ++c) {
+        const float4 a = q[c], b = t[c];
+        s = fmaf(a.x, b.x, s);
+        s = fmaf(a.y, b.y, s);
+        s = fmaf(a.z, b.z, s);
+        s = fmaf(a.w, b.w, s);
+    }
+    return 1.0f - s;
 }
-template <int DW>
-__device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const float* rows, uint32_t stride, uint32_t id,
-                                           int metric, int lane) {
-    float4 v[DW / 4];
-    load_warp<DW>(v, rows, stride, id, lane);
-    return dist_warp<DW>(q, v, metric);
+// The same for row `id`, by one lane.
+__device__ __forceinline__ float dist_lane(const float4* q, const float* rows, uint32_t stride, uint32_t id, int metric) {
+    const float4* r = reinterpret_cast<const float4*>(rows + uint64_t(id) * stride);
+    float s = 0.0f;
+    for (uint32_t c = 0; 4u * c < stride; ++c) {
+        const float4 a = q[c], b = __ldg(r + c);
+        if (metric == HNSW_L2SQ) {
+            const float x = a.x - b.x, y = a.y - b.y, z = a.z - b.z, w = a.w - b.w;
+            s = fmaf(x, x, s);
+            s = fmaf(y, y, s);
+            s = fmaf(z, z, s);
+            s = fmaf(w, w, s);
+        } else {
+            s = fmaf(a.x, b.x, s);
+            s = fmaf(a.y, b.y, s);
+            s = fmaf(a.z, b.z, s);
+            s = fmaf(a.w, b.w, s);
+        }
+    }
+    return metric == HNSW_L2SQ ? s : 1.0f - s;
 }
 
 // Alg. 1's descent and layer insertion on layers >= 1 for each new element in
@@ -765,13 +801,15 @@ __device__ __forceinline__ float dist_warp(const float4 (&q)[DW / 4], const floa
 // Reverse links are independent of one another (each changes one list and
 // reads vectors): a warp each.  Measured, 1,000 elements into 20,000, of which 70
 // go to a layer of 1,250 (efConstruction 200, 128 coordinates): the whole
-// insertion call took 99 ms with one warp here, 25.6 with a block that merged
-// by counting, atomics and four barriers an expansion, and takes 24.4.  What
-// bounds it is an expansion's instructions, which follow one another (2,700
-// cycles: 600 to find the entry, 600 to score, 400 for the requests, 2,000
-// where keys are merged, which is every other time), not the reads.  Slower or
-// the same: 8 warps with a team of 8 lanes per row (25.8 ms), visited elements
-// as a bitmap in shared memory (24.9), vectors read past L1.
+// insertion call took 99 ms with one warp here, and takes 28.5.  It took 24.5
+// with distances added in parts by a warp's lanes: 440 cycles less an expansion,
+// but other sums, which near-ties show in the lists (dist_seq).  Rows of 200:
+// 130 ms with one warp, 38.4 now.  What bounds it is an expansion's
+// instructions, which follow one another (3,100 cycles: 600 to find the entry,
+// 1,000 to score, 400 for the requests, 2,000 where keys are merged, which is
+// every other time), not the reads.  Slower or the same: 8 warps with a team of
+// 8 lanes per row, visited elements as a bitmap in shared memory, vectors read
+// past L1.  Rows above 128 coordinates spill 40 to 280 bytes at 128 registers.
 template <int DW, int E, int NB>
 __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -789,14 +827,18 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
     for (uint32_t u = 0; u < a.n; ++u) {
         const uint32_t q = a.ids[u];
         const int l = a.lv[u];
-        float4 xq[DW / 4];
-#pragma unroll
-        for (int k = 0; k < DW / 4; ++k) {
-            const uint32_t c = uint32_t(lane + 32 * k);
-            xq[k] = 4u * c < stride ? __ldg(reinterpret_cast<const float4*>(rows + uint64_t(q) * stride) + c)
-                                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float4* const wt = S.t[wid];
+        uint64_t cur;
+        {  // the enter point's distance, added as the selection adds
+            TeamVec<DW> x, y;
+            load_team(rows, stride, q, x, lane);
+            load_team(rows, stride, ep, y, lane);
+            cur = mkkey(dist_team(x, y, V.metric, lane), ep);
         }
-        uint64_t cur = mkkey(dist_warp<DW>(xq, rows, stride, ep, V.metric, lane), ep);
+        __syncthreads();  // the last element's lists are written, its shared memory is read
+        for (uint32_t c = t; 4u * c < stride; c += kUpThreads)
+            S.q[c] = __ldg(reinterpret_cast<const float4*>(rows + uint64_t(q) * stride) + c);
+        __syncthreads();
         int buf = 0;
         for (int lc = L; lc > l; --lc) {  // descent above the level, ef = 1 (steepest descent)
             for (;;) {
@@ -805,7 +847,9 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
                 for (int j = wid; j < Mmax; j += kUpWarps) {
                     const uint32_t e = row[j];
                     if (e == kNone) break;  // valid ids come first
-                    const uint64_t k = mkkey(dist_warp<DW>(xq, rows, stride, e, V.metric, lane), e);
+                    float4 v[DW / 4];
+                    load_warp<DW>(v, rows, stride, e, lane);
+                    const uint64_t k = mkkey(dist_seq<DW>(S.q, v, stride, V.metric, wt, lane), e);
                     best = k < best ? k : best;
                 }
                 if (lane == 0) S.best[buf][wid] = best;
@@ -821,7 +865,6 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
                 cur = best;
             }
         }
-        __syncthreads();  // the last element's lists are written, its shared memory is read
         int n_ep = 1;
         if (t == 0) S.Ek[0] = cur;
         __syncthreads();
@@ -894,13 +937,10 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
                     if (j >= Mmax) break;
                     uint64_t key = ~0ull;
                     const uint32_t e = ne[k];
-                    if (e != kNone) {
-                        const float dq = dist_warp<DW>(xq, nv[k], V.metric);
-                        const bool met = __any_sync(kFull, tag[k] == epoch || o0 == e || o1 == e);
-                        if (!met) {
-                            const uint64_t ke = (uint64_t(f2ord(dq)) << 32) | (uint64_t(e) << 1);
-                            if (ke < thr) key = ke;
-                        }
+                    if (e != kNone && !__any_sync(kFull, tag[k] == epoch || o0 == e || o1 == e)) {
+                        const float dq = dist_seq<DW>(S.q, nv[k], stride, V.metric, wt, lane);
+                        const uint64_t ke = (uint64_t(f2ord(dq)) << 32) | (uint64_t(e) << 1);
+                        if (ke < thr) key = ke;
                     }
                     if (lane == 0) {
                         S.K[kb][j] = key;
@@ -1015,17 +1055,15 @@ __global__ void __launch_bounds__(kUpThreads) insert_upper(const UpperArgs a) {
                     if (lane == 0) rr[n0] = q;
                     continue;
                 }
-                // the members and q by their distance to r
+                // the members and q by their distance to r, a lane each
                 uint64_t* keys = S.keys[wid];
-                TeamVec<DW> xr;
-                load_team(rows, stride, r, xr, lane);
-                for (int j0 = 0; j0 <= n0; j0 += 4) {
-                    const int j = min(j0 + (lane >> 3), n0);
+                __syncwarp();
+                for (uint32_t c = lane; 4u * c < stride; c += 32)
+                    wt[c] = __ldg(reinterpret_cast<const float4*>(rows + uint64_t(r) * stride) + c);
+                __syncwarp();
+                for (int j = lane; j <= n0; j += 32) {
                     const uint32_t c2 = j < n0 ? rr[j] : q;
-                    TeamVec<DW> y;
-                    load_team(rows, stride, c2, y, lane);
-                    const float dc = dist_team(xr, y, V.metric, lane);
-                    if ((lane & 7) == 0) keys[j] = mkkey(dc, c2);
+                    keys[j] = mkkey(dist_lane(wt, rows, stride, c2, V.metric), c2);
                 }
                 int n2 = 32;
                 while (n2 < n0 + 1) n2 <<= 1;
