@@ -208,6 +208,18 @@ __global__ void __launch_bounds__(kThreads) stop_fwd_bwd(const float* __restrict
                 const float y = S.y[b];
                 l = fmaxf(z, 0.0f) - z * y + log1pf(expf(-fabsf(z)));
                 dz = (1.0f / (1.0f + expf(-z)) - y) * scale;
+            } else {
+                // a place past the last sample holds the network's answer to
+                // zeros: cleared, so that the sums below add nothing for it
+                // (zero times an infinite weight would be NaN)
+                const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; i += 4) {
+                    *reinterpret_cast<float4*>(S.a2 + b * kLd + u0 + i) = none;
+                    *reinterpret_cast<float4*>(S.h1 + b * kLd + u0 + i) = none;
+                }
             }
             if ((t & 7) == 0) {
                 S.dz[b] = dz;
