@@ -151,7 +151,8 @@ bool on_gpu(const uint8_t* p, uint64_t n, cudaStream_t s, uint64_t& out) {
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
     const uint64_t pieces = n / kPiece;
     const uint64_t most = pieces < uint64_t(kChunkPieces) ? pieces : uint64_t(kChunkPieces);
-    keep_pool_memory();
+    // from the pool as the process has set it up: by default the memory goes
+    // back at the synchronisation below
     void* scr = nullptr;
     if (cudaMallocAsync(&scr, 2 * most * kPiece + 256 + most, s) != cudaSuccess) return false;
     uint8_t* data = static_cast<uint8_t*>(scr);

@@ -128,8 +128,6 @@ hnsw_status upload_index(const void* graph_blob, uint64_t blob_bytes, hnsw_dtype
 // fnv1a64 of n bytes of host memory, on the GPU where that is quicker (the
 // stream's work up to here is then waited for).
 uint64_t checksum64(const uint8_t* p, uint64_t n, cudaStream_t s);
-// Lets the device's default pool keep a bounded amount of freed memory.
-void keep_pool_memory();
 // Writes stored rows [first, first + n) (and the fp32 copy when kept) from
 // fp32 rows in device memory, d_pad32 floats apart; asynchronous on s.
 hnsw_status store_rows(hnsw_index* ix, const float* rows32, uint64_t first, uint64_t n, cudaStream_t s);
