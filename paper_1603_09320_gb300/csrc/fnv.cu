@@ -31,7 +31,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr uint64_t kPrime = 0x100000001b3ull;
 constexpr int kSub = 256;                 // bytes of a lane
 constexpr int kPiece = 32 * kSub;         // bytes of a warp
-constexpr int kChunkPieces = 2048;        // 16 MB of input, and as much for the maps
+constexpr int kChunkPieces = 2048;        // 16 MB of input
+constexpr int kMaps = 32 * 128;           // bytes of a piece's maps, 128 for every kSub of it
 constexpr int kBatch = 256;               // pieces whose maps fnv_starts holds at a time
 constexpr int kWarps = 4;
 
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(kWarps * 32) fnv_maps(const uint4* __restrict_
     const uint32_t piece = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (piece >= pieces) return;
     const uint4* in = data + uint64_t(piece) * (kPiece / 16);
-    uint32_t* out = maps + uint64_t(piece) * 32 * 32;
+    uint32_t* out = maps + uint64_t(piece) * (kMaps / 4);
     uint32_t a = uint32_t(lane) | uint32_t(lane + 32) << 16, b = uint32_t(lane + 64) | uint32_t(lane + 96) << 16;
     uint4 next = __ldg(in);
     for (int sub = 0; sub < 32; ++sub) {
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(kBatch) fnv_starts(const uint32_t* __restrict_
         const int n = int(min(uint32_t(kBatch), pieces - base));
         __syncthreads();
         for (int i = threadIdx.x; i < n * 32; i += kBatch)
-            m[i >> 5][i & 31] = maps[(uint64_t(base) + (i >> 5)) * 1024 + 31 * 32 + (i & 31)];
+            m[i >> 5][i & 31] = maps[(uint64_t(base) + (i >> 5)) * (kMaps / 4) + 31 * 32 + (i & 31)];
         __syncthreads();
         if (threadIdx.x == 0)
             for (int i = 0; i < n; ++i) {
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kWarps * 32) fnv_pieces(const uint4* __restric
     const uint32_t piece = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (piece >= pieces) return;
     uint32_t l = starts[piece];
-    if (lane > 0) l = follow(maps + (uint64_t(piece) * 32 + uint32_t(lane - 1)) * 128, l);
+    if (lane > 0) l = follow(maps + uint64_t(piece) * kMaps + uint32_t(lane - 1) * 128, l);
     const uint4* in = data + uint64_t(piece) * (kPiece / 16) + lane * (kSub / 16);
     uint64_t h = l;
     for (int i = 0; i < kSub / 16; ++i) {
@@ -154,11 +155,11 @@ bool on_gpu(const uint8_t* p, uint64_t n, cudaStream_t s, uint64_t& out) {
     // from the pool as the process has set it up: by default the memory goes
     // back at the synchronisation below
     void* scr = nullptr;
-    if (cudaMallocAsync(&scr, 2 * most * kPiece + 256 + most, s) != cudaSuccess) return false;
+    if (cudaMallocAsync(&scr, most * (kPiece + kMaps) + 256 + most, s) != cudaSuccess) return false;
     uint8_t* data = static_cast<uint8_t*>(scr);
     uint8_t* maps = data + most * kPiece;
-    FnvState* st = reinterpret_cast<FnvState*>(maps + most * kPiece);
-    uint8_t* starts = maps + most * kPiece + 256;
+    FnvState* st = reinterpret_cast<FnvState*>(maps + most * kMaps);
+    uint8_t* starts = maps + most * kMaps + 256;
     FnvState host{kFnvBasis, uint32_t(kFnvBasis & 0xffu)};
     cudaError_t e = cudaMemcpyAsync(st, &host, sizeof(host), cudaMemcpyHostToDevice, s);
     for (uint64_t at = 0; at < pieces && e == cudaSuccess; at += most) {
