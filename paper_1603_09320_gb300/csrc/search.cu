@@ -41,6 +41,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <utility>
 
 #include "common.hpp"
 #include "index.cuh"
@@ -153,14 +154,18 @@ int ceil_log2(uint64_t x) {
     return r;
 }
 
+int current_device() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev;
+}
+
 // Blocks of `threads` threads and `smem` bytes of kernel fn resident per SM
 // (negative: the query failed).  Cached per (device, kernel, threads, size).
 int blocks_per_sm(KernelFn fn, int threads, size_t smem) {
     static std::mutex mu;
     static std::map<std::tuple<int, const void*, int, size_t>, int> cache;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, reinterpret_cast<const void*>(fn), threads, smem);
+    const auto key = std::make_tuple(current_device(), reinterpret_cast<const void*>(fn), threads, smem);
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
@@ -174,9 +179,8 @@ int blocks_per_sm(KernelFn fn, int threads, size_t smem) {
 }
 
 int sm_count() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, current_device());
     return sms;
 }
 
@@ -185,8 +189,22 @@ int sm_count() {
 // block among equals: finer-grained blocks), and the blocks per SM then.
 // Small per-warp state is bound by registers (4-warp blocks); a wide beam's
 // state is bound by shared memory, where the block size decides how much of
-// an SM's 228 KB the blocks fill.
+// an SM's 228 KB the blocks fill.  Cached per (device, kernel, size): a launch
+// with an automatic visited set asks for up to six sizes (without this, eight
+// look-ups for each: 1 to 4 us of a call).
 bool block_choice(KernelFn fn, size_t warp_smem, int& warps, int& per_sm) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void*, size_t>, std::pair<int, int>> cache;
+    const auto key = std::make_tuple(current_device(), reinterpret_cast<const void*>(fn), warp_smem);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = cache.find(key);
+        if (it != cache.end()) {
+            warps = it->second.first;
+            per_sm = it->second.second;
+            return true;
+        }
+    }
     int best = 0;
     warps = 0;
     per_sm = 0;
@@ -201,7 +219,10 @@ bool block_choice(KernelFn fn, size_t warp_smem, int& warps, int& per_sm) {
             per_sm = b;
         }
     }
-    return best != 0;
+    if (best == 0) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    cache[key] = {warps, per_sm};
+    return true;
 }
 
 // The instantiation for an index's stored rows (null: none).
