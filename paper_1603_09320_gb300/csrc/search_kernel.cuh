@@ -99,23 +99,27 @@ HNSW_STOP_FN float stop_check(const StopDev* model, const uint64_t* W, int size,
     return model ? stop_logit<true>(model, f, hs, lane) : 0.0f;
 }
 
-// Register budget of each instantiation (per thread), where the kernel fits
-// without spilling: 56 -- 9 blocks of 128 threads resident per SM, 36 warps
-// -- for the 2-lane teams of low-d rows; 72 for fp32 rows of 128 coordinates
-// (80 with the stop, the bounds checks or partial rows); more for more rows in
-// flight (fp8 with 8 rows per team, f16 with 4); 64 (8 blocks) otherwise.  Full
-// bf16 rows at 56 registers spill 20 bytes and run slower in spite of 4 more
-// warps (10,000 queries at ef 50: 543 us against 520; low-d rows at 64: 1,047
-// against 989).  Without an explicit budget the compiler chose budgets that
-// spilled.  Blocks of up to 256 threads are allowed so that large per-warp
-// state (wide beams) can be packed into the shared memory of an SM (see the
-// launch).
-template <int ST, int TEAM, int CPL, int U, bool FULL, bool STOP, bool CHECK>
+// Register budget of each instantiation (per thread): 56 -- 9 blocks of 128
+// threads resident per SM, 36 warps -- for the 2-lane teams of low-d rows, but
+// for narrow searches with the stop on rows of one chunk, which spill 52 to 80
+// bytes at 56 (8 bf16 coordinates, 10,000 queries at ef 50: 329 us at 56, 285
+// at 64); 72 for fp32 rows of 128 coordinates (80 with the stop, the bounds
+// checks or partial rows); more for more rows in flight (fp8 with 8 rows per
+// team, f16 with 4); 64 (8 blocks) otherwise.  Full bf16 rows at 56 registers
+// spill 20 bytes and run slower in spite of 4 more warps (10,000 queries at ef
+// 50: 543 us against 520; low-d rows at 64: 1,047 against 989).  Partial fp32
+// rows spill 4 to 32 bytes at 80, and are quicker so than with fewer warps: 100
+// coordinates, 10,000 queries at ef 128, 717 us at 80, 805 at 88 without a
+// spill (ef 50: the same).  Without an explicit budget the compiler chose
+// budgets that spilled.  Blocks of up to 256 threads are allowed so that large
+// per-warp state (wide beams) can be packed into the shared memory of an SM
+// (see the launch).
+template <int ST, int TEAM, int CPL, int U, bool FULL, bool STOP, bool WIDE, bool CHECK>
 constexpr int search_max_regs() {
     return (ST == HNSW_F32 && CPL == 4) ? ((STOP || CHECK || !FULL) ? 80 : 72)
          : (ST == HNSW_FP8E4M3 && U == 8) ? 96
          : (ST == HNSW_F16 && U == 4) ? 80
-         : (TEAM == 2 && !CHECK) ? 56
+         : (TEAM == 2 && !CHECK && !(STOP && !FULL && !WIDE)) ? 56
                                  : 64;
 }
 
@@ -127,12 +131,12 @@ constexpr int search_max_regs() {
 // WIDE: launches whose W may hold more than 64 entries, or whose layer-0
 // lists more than 32 (merge_wide).
 template <int ST, int TEAM, int CPL, int U, bool FULL, bool STOP, bool WIDE, bool CHECK = false>
-__global__ void __launch_bounds__(256) __maxnreg__((search_max_regs<ST, TEAM, CPL, U, FULL, STOP, CHECK>()))
+__global__ void __launch_bounds__(256) __maxnreg__((search_max_regs<ST, TEAM, CPL, U, FULL, STOP, WIDE, CHECK>()))
     hnsw_search_kernel(const SearchArgs a) {
     using D = Dist<ST, TEAM, CPL, U, FULL>;
     // full fp32 rows of 128 coordinates have no registers left for the wide
     // merge's ballots at 72 (56 bytes of spill, 5% slower at ef 66 to 100)
-    constexpr bool kBallot = search_max_regs<ST, TEAM, CPL, U, FULL, STOP, CHECK>() != 72;
+    constexpr bool kBallot = search_max_regs<ST, TEAM, CPL, U, FULL, STOP, WIDE, CHECK>() != 72;
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     uint8_t* wbase = smem + (threadIdx.x >> 5) * a.warp_smem;
