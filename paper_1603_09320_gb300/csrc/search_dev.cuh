@@ -491,12 +491,14 @@ __device__ __forceinline__ bool visit_new(uint32_t* H, int hlog, uint32_t id, ui
 // that received a new key (INT_MAX: none did); ok stays set in the lanes whose
 // key is now in W.
 
-// W of at most 64 entries.  Every surviving key finds its lower bound in W by
+// W of at most 64 entries, or up to kNarrow ones of a longer beam's W (whose
+// lower bounds reach 63).  Every surviving key finds its lower bound in W by
 // ballots (few candidates) or a binary search of its own; one pass over the
 // survivors then gives each its rank among them (its final position is lower
 // bound + rank) and each W entry the number of survivors placed before it; W
 // is read into registers (entries lane and lane + 32) before any write, and
 // every entry is written once.
+constexpr int kNarrow = 63;
 __device__ __forceinline__ int merge_small(uint64_t* W, int& size, int efp, uint64_t k, bool& ok, int lane) {
     // W's entries lane and lane + 32 (beyond size: all ones, above every key)
     const uint64_t w0 = lane < size ? W[lane] : ~0ull;
@@ -579,7 +581,11 @@ __device__ __forceinline__ int merge_small(uint64_t* W, int& size, int efp, uint
 // per chunk whatever the number of new keys.  (The form that counted, for every
 // entry, the new keys placed before it took a pass over the new keys per
 // chunk: GloVe-shaped 400k, 10,000 queries at ef 498: 7.19 ms, 5.85 ms with
-// this merge and the shorter row distances.)
+// this merge and the shorter row distances.  A single new key needs no
+// bitmap.  That, and merge_small while W is short, is for beams just above 64
+// entries, where most of a search is W's growth and single keys: SIFT-shaped 1M,
+// 1,200 queries at ef 66, f16 rows 542 us without, 532 with, fp32 550 / 536 (a
+// list of new keys per chunk: 529 / 535).
 template <bool BALLOT>
 __device__ __forceinline__ int merge_wide(uint64_t* W, int& size, int efp, uint64_t k, bool& ok, int lane) {
     const uint64_t wlast = size > 0 ? (W[size - 1] >> 1) : 0ull;
@@ -612,10 +618,23 @@ __device__ __forceinline__ int merge_wide(uint64_t* W, int& size, int efp, uint6
     }
     const uint32_t surv = __ballot_sync(kFull, ok);
     if (surv == 0) return INT_MAX;
-    int pos = lb;
-    if (surv & (surv - 1)) {
-        for (uint32_t bits = surv; bits; bits &= bits - 1) pos += __shfl_sync(kFull, k1, __ffs(bits) - 1) < k1;
+    if (!(surv & (surv - 1))) {  // one new key, the common case in a full W: its place is known
+        const int p = __shfl_sync(kFull, lb, __ffs(surv) - 1);
+        const int nsize = min(efp, size + 1);
+        for (int c = (nsize - 1) >> 5; c >= p >> 5; --c) {
+            const int t = c * 32 + lane;
+            const bool mv = t > p && t < nsize;
+            const uint64_t v = mv ? W[t - 1] : 0ull;
+            __syncwarp();  // a chunk's reads precede its writes
+            if (mv) W[t] = v;
+        }
+        if (ok) W[p] = k;
+        size = nsize;
+        __syncwarp();
+        return p;
     }
+    int pos = lb;
+    for (uint32_t bits = surv; bits; bits &= bits - 1) pos += __shfl_sync(kFull, k1, __ffs(bits) - 1) < k1;
     ok = ok && pos < efp;
     const uint32_t in = __ballot_sync(kFull, ok);  // not empty: the smallest survivor is below W's last entry
     const int first = int(__reduce_min_sync(kFull, ok ? uint32_t(pos) : 0xffffffffu));

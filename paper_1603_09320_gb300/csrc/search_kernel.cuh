@@ -395,8 +395,9 @@ __global__ void __launch_bounds__(256) __maxnreg__((search_max_regs<ST, TEAM, CP
                         const int j = h + lane;
                         bool ok = j < n;
                         const uint64_t key = ok ? mkkey(dst[j], ids[j]) : 0ull;
-                        first_new = min(first_new, WIDE ? merge_wide<kBallot>(W, size, efq, key, ok, lane)
-                                                        : merge_small(W, size, efq, key, ok, lane));
+                        first_new = min(first_new, WIDE && (CHECK || size > kNarrow)
+                                                   ? merge_wide<kBallot>(W, size, efq, key, ok, lane)
+                                                   : merge_small(W, size, efq, key, ok, lane));
                     }
                 }
                 scan = min(p + 1, first_new);
