@@ -354,10 +354,11 @@ struct Dist {
         return acc;
     }
 
-    // run() where the warp takes one row of several chunks per lane at a time
-    // (fp32 rows above 128 coordinates): written out so that the reads of two
-    // rows overlap (200 coordinates, 10,000 queries at ef 50: 854 us a row after
-    // another, 810 so)
+    // run() where the warp takes one row at a time (rows above 128 coordinates):
+    // written out so that the reads of two rows overlap (10,000 queries at ef
+    // 50, a row after another / so: 200 fp32 coordinates 854 / 810 us, 256 bf16
+    // 687 / 649, 256 fp8 735 / 722; the fp8 instances with the stop then spill 8
+    // to 40 bytes and are as quick or quicker all the same)
     __device__ static void run_row_pairs(const DevIndex& ix, const float (&qr)[QF], const uint32_t* ids, int n,
                                          float* out, int lane) {
         const uint32_t C = ix.row_chunks;
@@ -371,7 +372,9 @@ struct Dist {
                 const uint32_t ch = uint32_t(lane + c * 32);
                 v[c] = FULL || ch < C ? ld_row_chunk(rowp + ch) : make_uint4(0u, 0u, 0u, 0u);
             }
-            float acc = share(qr, v, 0.0f, l2);
+            float sc = 0.0f;
+            if (ST == HNSW_FP8E4M3) sc = __ldg(ix.scale + ids[r]);
+            float acc = share(qr, v, sc, l2);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
             if (lane == 0) out[r] = l2 ? acc : 1.0f - acc;
@@ -390,7 +393,7 @@ struct Dist {
     // plain reductions, 520 / 575 us with joint ones.
     __device__ static void run(const DevIndex& ix, const float (&qr)[QF], const uint32_t* ids, int n,
                                float* out, int lane) {
-        if constexpr (ST == HNSW_F32 && TEAM == 32 && U == 1) {
+        if constexpr (TEAM == 32 && U == 1) {
             run_row_pairs(ix, qr, ids, n, out, lane);
             return;
         }
