@@ -289,12 +289,15 @@ enum class Defer { no, automatic, always };
 // keep more of W in registers and shared memory: three 4-warp blocks (ef 498,
 // warp per query / block: 400 queries 1.24 times the time, 608 on GloVe-shaped
 // data 0.83 to 0.88 times).  Rows of up to 32 bytes leave little to score
-// ahead: with beams above 64 and no rerank a warp per query is as quick or
-// quicker (8 fp32 coordinates, ef 200, 8 to 60 queries: 0.86 to 0.96 times).
+// ahead: without rerank a warp per query is as quick or quicker above ef 64 (8
+// fp32 coordinates, ef 200, 8 queries: block 298 us, warp 266), with rerank
+// above ef 256 (8 f16 coordinates, block / warp: ef 257, 40 queries 559 / 464,
+// 400 queries 842 / 755; ef 498, 400 queries 1,300 / 1,246; but ef 256, 77
+// queries 448 / 513).
 int team_warps(const DevIndex& D, const hnsw_search_params& p, uint32_t n) {
     const int efp = std::max(p.ef, p.k);
     if (p.schedule != 0 || p.check_bounds || D.N == 0 || D.N >= kTeamMaxN || efp > 512) return 0;
-    if (D.row_chunks <= 2 && efp > 64 && !p.rerank) return 0;
+    if (D.row_chunks <= 2 && efp > (p.rerank ? 256 : 64)) return 0;
     const uint32_t sms = uint32_t(sm_count());
     return n <= 2 * sms ? 8 : n <= (efp > 256 ? 3 : 4) * sms ? 4 : 0;
 }
