@@ -179,8 +179,13 @@ KernelFn search_kernel_fp8(const KernelAsk& k);
 
 // ---- keys -----------------------------------------------------------------
 // key = ord(dist) << 32 | id << 1 | expanded.  key >> 1 orders (dist, id).
+// The bits are taken by an instruction of its own: where the compiler sees that
+// f is a sum of squares it takes the sign bit for clear and makes the flip a
+// float negation, which gives a NaN back without its sign -- a key below all
+// others instead of above them, and a distance of -0.
 __device__ __forceinline__ uint32_t f2ord(float f) {
-    const uint32_t b = __float_as_uint(f);
+    uint32_t b;
+    asm("mov.b32 %0, %1;" : "=r"(b) : "f"(f));
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 __device__ __forceinline__ float ord2f(uint32_t o) {
