@@ -241,7 +241,12 @@ hnsw_status hnsw_search(hnsw_index* index, const float* queries, int64_t n, int3
 /* Per-query counters (the paper's cost measure is the number of distance
  * computations, Section 5.1). */
 typedef struct {
-    uint32_t n_eval;    /* distance evaluations on all layers */
+    uint32_t n_eval;    /* distance evaluations that the search asked for, on all layers:
+                           the neighbours met outside the visited set (repeats of elements
+                           it forgot among them), and the enter point.  Rows that the
+                           small-batch search scored ahead and did not need, and the
+                           rerank's rows, are not counted.  With flag bit 0 set the count
+                           of a small batch may differ from run to run */
     uint32_t n_exp0;    /* layer-0 expansions (elements taken from C) */
     uint32_t n_stepU;   /* elements expanded on layers >= 1 */
     uint32_t flags;     /* bit0: visited set overflowed (lossy, results unaffected);
@@ -259,19 +264,25 @@ typedef struct {
     int32_t visited_log2;    /* log2 of visited-set slots per query; 0 = automatic: the
                                 largest set from 2^8 up to 8-16 slots per beam entry
                                 (at most 2^12) that keeps as many warps resident as
-                                2^8 slots do (the set may forget elements, which only
-                                repeats evaluations; results are the same at any size) */
+                                2^8 slots do, for small batches (schedule 0) up to 64-128
+                                slots per beam entry (2^10 to 2^14) as long as as many
+                                queries are resident (the set may forget elements, which
+                                only repeats evaluations; results are the same at any
+                                size) */
     float stop_threshold;    /* learned stop: in (0,1) stop the layer-0 beam when the stop
                                 network's sigmoid exceeds it (needs hnsw_set_stop_model);
                                 <= 0 or >= 1: off, the plain search */
     int32_t stop_period;     /* learned stop / trace: check every stop_period layer-0
                                 expansions (<= 0: 8 for the stop, 4 for traces;
                                 above 65535: HNSW_EINVAL) */
-    int32_t schedule;        /* order of the work (results and counters unchanged; both
-                                scheduled forms take stream-ordered scratch, 16 bytes per
-                                query):
-                                0: automatic -- deferral (3) for batches of 33 to 2^24
-                                queries, else one pass;
+    int32_t schedule;        /* order of the work (results, n_exp0 and n_stepU unchanged,
+                                n_eval but for repeats; both scheduled forms, 2 and 3,
+                                take stream-ordered scratch, 16 to 20 bytes per query):
+                                0: automatic -- a block of warps per query while that
+                                leaves every query resident at once (up to 2 to 4 queries
+                                per SM, ef' up to 512; no scratch); deferral (3) for
+                                batches of 33 to 2^24 queries that give some warp several
+                                of them; else one pass;
                                 1: one pass in input order;
                                 2: two passes -- the upper-layer descent of all queries
                                 first, then the layer-0 beams in order of decreasing

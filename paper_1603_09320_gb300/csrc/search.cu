@@ -1,7 +1,8 @@
 // search.cu -- batched K-NN-SEARCH (arXiv:1603.09320, Alg. 5) on one GPU.
 //
 // One warp answers one query at a time; warps pull query indexes from a
-// device work counter until the batch is exhausted (persistent kernel).
+// device work counter until the batch is exhausted (persistent kernel).  Small
+// batches take a block of warps per query (search_team.cuh; team_warps below).
 //
 // Per query:
 //   1. greedy ef=1 descent through layers L..1 (Alg. 5's descent).  Under key
@@ -24,10 +25,12 @@
 // Visited set: a 4-way bucketed hash of element ids in shared memory; when a
 // bucket is full one of its slots is overwritten, and two lanes storing into
 // the same free slot at the same instant keep only one id, so the set may
-// FORGET an element.  Forgetting never changes
-// the result: an element met again is either already in W (its key equals an
-// entry's key and the merge drops it) or, being outside W after it was
-// visited, has a key above the furthest entry of a full W and is rejected.
+// FORGET an element.  (The block-per-query kernel tries eight buckets before it
+// overwrites, and stores again what it lost to another lane: search_team.cuh,
+// visit_all.)  Forgetting never changes the result: an element met again is
+// either already in W (its key equals an entry's key and the merge drops it)
+// or, being outside W after it was visited, has a key above the furthest entry
+// of a full W and is rejected.
 // It only costs a repeated distance evaluation, counted in n_eval.
 //
 // Distances: each row is read as 16-byte chunks by a team of TEAM lanes
@@ -645,8 +648,9 @@ extern "C" hnsw_status hnsw_search_ex(hnsw_index* ix, const hnsw_search_params* 
         sm.period = p->stop_period > 0 ? p->stop_period : 8;
         smp = &sm;
     }
-    // schedule: 0 automatic (deferral for 33 to 2^24 queries, else one pass),
-    // 1 one pass in input order, 2 two passes, 3 deferral
+    // schedule: 0 automatic (a block per query for small batches; deferral for
+    // 33 to 2^24 queries that give some warp several; else one pass), 1 one
+    // pass in input order, 2 two passes, 3 deferral
     const DevIndex snap = dev_snapshot(ix);  // both passes search the same version
     const bool two = snap.N > 0 && !p->check_bounds && p->schedule == 2;
     const Defer defer = snap.N == 0 || p->check_bounds ? Defer::no

@@ -1,5 +1,5 @@
 // search_dev.cuh -- device code shared by the search kernels (search.cu: one
-// warp per query; search_team.cu: a block per query): launch arguments, keys,
+// warp per query; search_team.cuh: a block per query): launch arguments, keys,
 // row decoding and distances, the visited set, the merges into W, rerank.
 #pragma once
 
@@ -131,14 +131,14 @@ struct SearchArgs {
     float* tr_logit;     // [n][tr_max] (only with a model)
     int32_t* tr_count;   // [n] checks recorded
     int tr_max;
-    // two-pass scheduling: mode 0 = descent and beam per query in input order;
-    // mode 1 = descent only, writing the layer-0 enter key and the upper-layer
-    // counters of every query; mode 2 = beam only, queries taken in `order`
     // grouped launch (several requests in one launch): per-query k (low 16
     // bits) and ef (high 16 bits), and the first output slot of each query;
     // null: k, efp and qi * k for every query
     const uint32_t* q_kef;
     const uint64_t* q_out;
+    // two-pass scheduling: mode 0 = descent and beam per query in input order;
+    // mode 1 = descent only, writing the layer-0 enter key and the upper-layer
+    // counters of every query; mode 2 = beam only, queries taken in `order`
     int mode;
     uint64_t* ep_keys;   // [n]
     uint32_t* up_cnt;    // [n][2]: distance evaluations, rows read on layers >= 1
@@ -609,19 +609,19 @@ __device__ __forceinline__ int merge_small(uint64_t* W, int& size, int efp, uint
 }
 
 // W of up to 1,024 entries.  Lower bounds by ballots (BALLOT: where registers
-// are left for them) or binary search, ranks among the
-// survivors as above; the final positions of the new keys are then a bitmap
-// (one 32-bit word per lane: 1,024 positions); the count of its bits below a
-// position says where that position's entry comes from, so that W moves up in
-// one pass over its 32-entry chunks, top chunk first, with a few instructions
-// per chunk whatever the number of new keys.  (The form that counted, for every
-// entry, the new keys placed before it took a pass over the new keys per
-// chunk: GloVe-shaped 400k, 10,000 queries at ef 498: 7.19 ms, 5.85 ms with
-// this merge and the shorter row distances.  A single new key needs no
-// bitmap.  That, and merge_small while W is short, is for beams just above 64
-// entries, where most of a search is W's growth and single keys: SIFT-shaped 1M,
-// 1,200 queries at ef 66, f16 rows 542 us without, 532 with, fp32 550 / 536 (a
-// list of new keys per chunk: 529 / 535).
+// are left for them) or binary search, ranks among the survivors as above; the
+// final positions of the new keys are then a bitmap (one 32-bit word per lane:
+// 1,024 positions); the count of its bits below a position says where that
+// position's entry comes from, so that W moves up in one pass over its 32-entry
+// chunks, top chunk first, with a few instructions per chunk whatever the number
+// of new keys.  The form that counted, for every entry, the new keys placed
+// before it took a pass over the new keys per chunk: GloVe-shaped 400k, 10,000
+// queries at ef 498: 7.19 ms, 5.85 ms with this merge and the shorter row
+// distances.  A single new key needs no bitmap.  That, and merge_small while W
+// is short, is for beams just above 64 entries, where most of a search is W's
+// growth and single keys: SIFT-shaped 1M, 1,200 queries at ef 66, us with the
+// counting form / without these two / with them: f16 529 / 542 / 532, fp32 535 /
+// 550 / 536.
 template <bool BALLOT>
 __device__ __forceinline__ int merge_wide(uint64_t* W, int& size, int efp, uint64_t k, bool& ok, int lane) {
     const uint64_t wlast = size > 0 ? (W[size - 1] >> 1) : 0ull;

@@ -1,6 +1,6 @@
 // search_kernel.cuh -- the one-warp-per-query search kernel (described in
 // search.cu) and the choice of its instantiation; instantiated per storage
-// type in search_f32.cu, search_b16.cu and search_fp8.cu.
+// type in search_f32.cu, search_bf16.cu, search_f16.cu and search_fp8.cu.
 #pragma once
 
 #include "search_dev.cuh"
