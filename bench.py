@@ -488,12 +488,14 @@ def e2e_host(args, ix, setting, Q, steps):
 
 
 def kernel_source_sha():
-    """Hash of the search kernel's code (search.cu and its headers) with
-    comments and blank space removed, so that counters taken on a kernel stay
-    matched to it across comment edits."""
+    """Hash of the search kernel's code (its launch, its headers and the lists
+    of its instances) with comments and blank space removed, so that counters
+    taken on a kernel stay matched to it across comment edits.  A file that is
+    missing (renamed, say) counts as different code."""
     files = [os.path.join(ROOT, "paper_1603_09320_gb300", "csrc", f)
-             for f in ("search.cu", "search_kernel.cuh", "search_dev.cuh")]
-    src = "\n".join(open(f).read() for f in files if os.path.exists(f))
+             for f in ("search.cu", "search_kernel.cuh", "search_dev.cuh", "search_pick.cuh", "search_f32.cu",
+                       "search_bf16.cu", "search_f16.cu", "search_fp8.cu")]
+    src = "\n".join(open(f).read() if os.path.exists(f) else "missing: " + os.path.basename(f) for f in files)
     src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
     src = re.sub(r"//[^\n]*", " ", src)
     src = " ".join(src.split())
