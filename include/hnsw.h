@@ -192,8 +192,9 @@ hnsw_status hnsw_reserve(hnsw_index* index, uint64_t capacity, void* stream);
  * issue it on a stream created non-blocking (not the legacy default stream,
  * which would serialise the searches of other streams behind the call).
  * Errors: HNSW_EINVAL (null pointers, no reserved capacity, capacity or
- * upper rows exceeded, level_u outside (0,1], d > 256, fp32 vectors absent),
- * HNSW_ENOMEM, HNSW_ECUDA. */
+ * upper rows exceeded, level_u outside (0,1], d > 256, fp32 vectors absent, a
+ * graph whose header has M outside 1..min(Mmax, Mmax0) or efConstruction
+ * outside 1..1024), HNSW_ENOMEM, HNSW_ECUDA. */
 hnsw_status hnsw_insert(hnsw_index* index, const float* data, uint64_t n, const double* level_u, void* stream);
 
 /* The index's current graph as a library-allocated "HNSWGB01" blob (free

@@ -1215,6 +1215,8 @@ extern "C" hnsw_status hnsw_insert(hnsw_index* ix, const float* data, uint64_t n
     const int heur = (ix->build_flags & 1u) ? 1 : 0, keep = (ix->build_flags & 4u) ? 1 : 0;
     if ((ix->build_flags & 2u) != 0) return ins_fail(HNSW_EINVAL, "graphs built with extendCandidates");
     if (efc < 1 || efc > 1024) return ins_fail(HNSW_EINVAL, "efConstruction of the graph outside 1..1024");
+    // a list's rows and a selection's places are Mmax and Mmax0 (<= kMaxOld)
+    if (M < 1 || M > Mmax || M > Mmax0) return ins_fail(HNSW_EINVAL, "M of the graph outside 1..min(Mmax, Mmax0)");
     // levels (the level draw of Alg. 1) and the new upper rows, in id order
     std::vector<uint8_t> lv(n);
     std::vector<uint32_t> up(n, kNone), U, Z;
