@@ -110,8 +110,9 @@ HNSW_STOP_FN float stop_check(const StopDev* model, const uint64_t* W, int size,
 // 50: 543 us against 520; low-d rows at 64: 1,047 against 989).  Partial fp32
 // rows spill 4 to 32 bytes at 80, and are quicker so than with fewer warps: 100
 // coordinates, 10,000 queries at ef 128, 717 us at 80, 805 at 88 without a
-// spill (ef 50: the same).  Without an explicit budget the compiler chose
-// budgets that spilled.  Blocks of up to 256 threads are allowed so that large
+// spill (ef 50: the same).  Full fp32 rows with the stop and a wide W spill 8
+// bytes there.  Without an explicit budget the compiler chose budgets that
+// spilled.  Blocks of up to 256 threads are allowed so that large
 // per-warp state (wide beams) can be packed into the shared memory of an SM
 // (see the launch).
 template <int ST, int TEAM, int CPL, int U, bool FULL, bool STOP, bool WIDE, bool CHECK>
